@@ -248,10 +248,17 @@ SpmvArgs spmv_args(const hec_matrix_s *A)
 
 // CTAs of an SpMV launch: one per row block (one 512-row tile in FP64, two
 // in FP32, where a thread owns four rows), at most 8 per SM.
-int spmv_grid(const hec_matrix_s *A, bool fp32)
+// With fused FP64 dots a CTA also pays a block reduction, so past one wave the
+// CTAs take equal numbers of row blocks, at most 4 CTAs per SM.
+int spmv_grid(const hec_matrix_s *A, bool fp32, int ndot)
 {
     const int64_t tiles = (A->hec.n + kSpmvTile - 1) / kSpmvTile;
-    return grid_for(fp32 ? (tiles + 1) / 2 : tiles, 1, 8);
+    const int64_t blocks = fp32 ? (tiles + 1) / 2 : tiles;
+    const int grid = grid_for(blocks, 1, 8);
+    if (ndot == 0 || fp32 || grid == blocks)
+        return grid;
+    const int64_t per = (blocks + 4 * device_sms() - 1) / (4 * device_sms());
+    return (int)((blocks + per - 1) / per);
 }
 
 int run_spmv(const hec_matrix_s *A, SpmvArgs a, int mode, int ndot, cudaStream_t s,
@@ -261,7 +268,7 @@ int run_spmv(const hec_matrix_s *A, SpmvArgs a, int mode, int ndot, cudaStream_t
         a.ell_val = A->ell_val32.p;
         a.tail_val = A->tail_val32.p;
     }
-    if (launch_spmv(a, mode, ndot, !A->hec.tail_rows.empty(), spmv_grid(A, fp32), s, fp32) != 0)
+    if (launch_spmv(a, mode, ndot, !A->hec.tail_rows.empty(), spmv_grid(A, fp32, ndot), s, fp32) != 0)
         return fail(HEC_ERR_INVALID, "no SpMV variant for mode %d ndot %d", mode, ndot);
     return check_launch("spmv");
 }
@@ -286,9 +293,20 @@ int ensure_f32(hec_matrix_s *A, cudaStream_t s)
 
 int vec_grid(int64_t n) { return grid_for(n, kThreads, 8); }
 
+// CTAs of a streaming launch that also reduces in FP64: every CTA pays one block
+// reduction and one partial for the last CTA to add, so past one element a
+// thread on every SM a CTA takes several, up to 4 CTAs per SM.
+int reduce_grid(int64_t n)
+{
+    const int spread = grid_for(n, kThreads, 1);
+    return std::max(spread, grid_for(n, 4 * kThreads, 4));
+}
+
 int run_vec(VecOp op, const VecArgs &a, cudaStream_t s)
 {
-    if (launch_vec(op, a, vec_grid(a.n), s) != 0)
+    const bool reduces = op == V_DOT || op == V_NRM2SQ || op == V_BICG_S || op == V_BICG_XR ||
+                         op == V_CG_XR;
+    if (launch_vec(op, a, reduces ? reduce_grid(a.n) : vec_grid(a.n), s) != 0)
         return fail(HEC_ERR_INVALID, "bad vector op");
     return check_launch("vector op");
 }
@@ -844,7 +862,7 @@ int seq_gmres_step(hec_matrix_s *A, hec_precond_s *M, Solver &S, cudaStream_t cs
     w.y_out = S.w;
     w.op = FIN_GMRES_W0;
     HEC_TRY(run_spmv(A, w, 0, 1, cs, f)); // w = A z, ||w||
-    const int mdgrid = grid_for(n, kThreads, 2);
+    const int sms = device_sms();
     BasisArgs h{};
     h.n = n;
     h.k = m + 1;
@@ -855,7 +873,7 @@ int seq_gmres_step(hec_matrix_s *A, hec_precond_s *M, Solver &S, cudaStream_t cs
     h.red = S.red.r;
     h.st = S.st;
     h.op = FIN_GMRES_H1;
-    launch_multidot(h, mdgrid, cs, f); // h1 = V^T w
+    launch_multidot(h, sms, cs, f); // h1 = V^T w
     HEC_TRY(check_launch("multidot"));
     BasisArgs up = h;
     up.coef = dev_field<double>(S.st, offsetof(SolverState, h1));
@@ -864,13 +882,13 @@ int seq_gmres_step(hec_matrix_s *A, hec_precond_s *M, Solver &S, cudaStream_t cs
     HEC_TRY(check_launch("basis update"));
     BasisArgs h2 = h;
     h2.op = FIN_GMRES_H2;
-    launch_multidot(h2, mdgrid, cs, f); // h2 = V^T w
+    launch_multidot(h2, sms, cs, f); // h2 = V^T w
     HEC_TRY(check_launch("multidot"));
     BasisArgs up2 = h;
     up2.coef = dev_field<double>(S.st, offsetof(SolverState, h2));
     up2.wout = S.w;
     up2.op = FIN_GMRES_STEP;
-    launch_basis_update(up2, true, vec_grid(n), cs, f); // w -= V h2, ||w||, Givens
+    launch_basis_update(up2, true, f ? vec_grid(n) : reduce_grid(n), cs, f); // w -= V h2, ||w||, Givens
     HEC_TRY(check_launch("basis update"));
     VecArgs sc{};
     sc.n = n;
@@ -1629,7 +1647,7 @@ int hec_multidot(int32_t n, int32_t k, const double *V, int64_t ldv, const doubl
         a.result = h;
         a.op = FIN_STORE;
         HEC_TRY(global_reducer(s, a.red));
-        launch_multidot(a, grid_for(n, kThreads, 2), s);
+        launch_multidot(a, device_sms(), s);
         return check_launch("multidot");
     });
 }

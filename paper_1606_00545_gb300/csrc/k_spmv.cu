@@ -102,7 +102,7 @@ __device__ __forceinline__ T warp_sum_t(T v)
 template <class T> constexpr int spmv_tiles_per_block() { return RowVec<T>::RPT / 2; }
 
 template <int MODE, int NDOT, bool TAIL, class T>
-__global__ void __launch_bounds__(kThreads) k_spmv_hec(SpmvArgs a)
+__global__ void __launch_bounds__(kThreads, TAIL ? 1 : NDOT > 0 ? 6 : 8) k_spmv_hec(SpmvArgs a)
 {
     using RV = RowVec<T>;
     constexpr int RPT = RV::RPT, TPB = RPT / 2, BR = kThreads * RPT;
@@ -110,10 +110,17 @@ __global__ void __launch_bounds__(kThreads) k_spmv_hec(SpmvArgs a)
     if (a.st && a.st->skip)
         return; // uniform across the grid: set before this launch
     __shared__ T s_tail[TAIL ? BR : 1];
-    T acc[NDOT > 0 ? NDOT : 1];
+    // The dots' per-thread sums live in shared memory between row blocks:
+    // with them in registers the kernel takes 42, 5 CTAs per SM, and the
+    // gathers' latency is less well hidden.  At 40 registers, 6 CTAs per SM
+    // and 4 per SM launched (see spmv_grid), the 128^3 SpMV with two dots
+    // takes 46 us (61 before, 32 without dots; the FP64 pipe alone needs 30
+    // for its 9 multiply-adds a row).  8 CTAs per SM spill: 47-51 us; the
+    // dots' partners loaded ahead of the slab: 56 us.
+    __shared__ T s_acc[NDOT > 0 ? NDOT : 1][NDOT > 0 ? kThreads : 1];
 #pragma unroll
-    for (int d = 0; d < (NDOT > 0 ? NDOT : 1); ++d)
-        acc[d] = T(0);
+    for (int d = 0; d < NDOT; ++d)
+        s_acc[d][threadIdx.x] = T(0);
     const typename RV::V *__restrict__ valv = reinterpret_cast<const typename RV::V *>(a.ell_val);
     const typename RV::C *__restrict__ colv = reinterpret_cast<const typename RV::C *>(a.ell_col);
     const T *__restrict__ x = reinterpret_cast<const T *>(a.x);
@@ -184,6 +191,7 @@ __global__ void __launch_bounds__(kThreads) k_spmv_hec(SpmvArgs a)
             for (int j = 0; j < RPT; ++j)
                 s[j] = T(0);
             const int p0 = r0 / RPT;
+            const int nr = min(RPT, a.n - r0); // rows of this thread inside the matrix
             const uint64_t pol = evict_first_policy();
 #pragma unroll 4
             for (int k = 0; k < a.K; ++k) {
@@ -193,7 +201,6 @@ __global__ void __launch_bounds__(kThreads) k_spmv_hec(SpmvArgs a)
                 for (int j = 0; j < RPT; ++j)
                     s[j] = fma(RV::get(v, j), __ldg(&x[RV::col(c, j)]), s[j]);
             }
-            const int nr = min(RPT, a.n - r0); // rows of this thread inside the matrix
             T y[RPT];
 #pragma unroll
             for (int j = 0; j < RPT; ++j) {
@@ -220,11 +227,13 @@ __global__ void __launch_bounds__(kThreads) k_spmv_hec(SpmvArgs a)
 #pragma unroll
             for (int d = 0; d < NDOT; ++d) {
                 const T *w = reinterpret_cast<const T *>(d == 0 ? a.w0 : a.w1);
+                T acc = s_acc[d][threadIdx.x];
 #pragma unroll
                 for (int j = 0; j < RPT; ++j) {
                     const T q = j < nr ? (w ? w[r0 + j] : y[j]) : T(0);
-                    acc[d] = fma(q, y[j], acc[d]);
+                    acc = fma(q, y[j], acc);
                 }
+                s_acc[d][threadIdx.x] = acc;
             }
         }
         if (TAIL)
@@ -234,7 +243,7 @@ __global__ void __launch_bounds__(kThreads) k_spmv_hec(SpmvArgs a)
         double v[NDOT];
 #pragma unroll
         for (int d = 0; d < NDOT; ++d)
-            v[d] = double(acc[d]);
+            v[d] = double(s_acc[d][threadIdx.x]);
         reduce_and_finalize<NDOT>(v, a.red, a.op, a.result, a.st);
     }
 }

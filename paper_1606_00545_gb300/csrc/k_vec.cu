@@ -61,57 +61,102 @@ __global__ void __launch_bounds__(kThreads) k_vec(VecArgs a)
         mode = st->s_conv ? 1 : (st->skip ? 2 : 0);
     }
 
-    const int stride = gridDim.x * kThreads;
-    for (int i = blockIdx.x * kThreads + threadIdx.x; i < a.n; i += stride) {
-        if (OP == V_AXPBY) {
-            z[i] = c0 * x[i] + c1 * z[i];
-        } else if (OP == V_WAXPBY) {
-            z[i] = c0 * x[i] + c1 * a.y[i];
+    // kUnroll elements per thread and pass, all their loads issued before the
+    // first store, so that enough bytes are in flight to stream from HBM
+    struct Elem {
+        double p0, p1, p2, p3, p4;
+    };
+    auto load = [&](int i) -> Elem {
+        Elem e{};
+        if (OP == V_AXPBY)
+            e = {x[i], z[i], 0, 0, 0};
+        else if (OP == V_WAXPBY || OP == V_DOT || OP == V_BICG_S)
+            e = {x[i], a.y[i], 0, 0, 0};
+        else if (OP == V_NRM2SQ || OP == V_COPY || OP == V_SCALE_ST)
+            e.p0 = x[i];
+        else if (OP == V_BICG_P) {
+            e.p0 = x[i];
+            if (!mode) {
+                e.p1 = a.y[i];
+                e.p2 = z[i];
+            }
+        } else if (OP == V_BICG_XR) {
+            if (mode == 0)
+                e = {a.w[i], a.u[i], a.v[i], a.q[i], x[i]};
+            else if (mode == 1)
+                e = {a.w[i], a.u[i], 0, 0, 0};
+        } else if (OP == V_CG_XR) {
+            if (!mode)
+                e = {a.w[i], a.u[i], a.q[i], z[i], 0};
+        } else if (OP == V_CG_P) {
+            e.p0 = x[i];
+            if (!mode)
+                e.p1 = z[i];
+        } else if (OP == V_AXPY_ST1)
+            e = {x[i], z[i], 0, 0, 0};
+        return e;
+    };
+    auto store = [&](int i, const Elem &e) {
+        if (OP == V_AXPBY || OP == V_WAXPBY) {
+            z[i] = c0 * e.p0 + c1 * e.p1;
         } else if (OP == V_DOT) {
-            acc[0] = fma(x[i], a.y[i], acc[0]);
+            acc[0] = fma(e.p0, e.p1, acc[0]);
         } else if (OP == V_NRM2SQ) {
-            double t = x[i];
-            acc[0] = fma(t, t, acc[0]);
+            acc[0] = fma(e.p0, e.p0, acc[0]);
         } else if (OP == V_COPY) {
-            z[i] = x[i];
+            z[i] = e.p0;
         } else if (OP == V_SCALE_ST) {
-            z[i] = c0 * x[i];
+            z[i] = c0 * e.p0;
         } else if (OP == V_BICG_P) {
             // x = r, y = v, z = p
-            z[i] = mode ? x[i] : fma(c0, z[i] - c1 * a.y[i], x[i]);
+            z[i] = mode ? e.p0 : fma(c0, e.p2 - c1 * e.p1, e.p0);
         } else if (OP == V_BICG_S) {
             // x = r, y = v, z = s
-            double s = fma(-c0, a.y[i], x[i]);
+            const double s = fma(-c0, e.p1, e.p0);
             z[i] = s;
             acc[0] = fma(s, s, acc[0]);
         } else if (OP == V_BICG_XR) {
             // w = x (solution), u = p*, v = s*, q = t, x = s, y = r0, z = r
             if (mode == 0) {
-                a.w[i] = fma(c1, a.v[i], fma(c0, a.u[i], a.w[i]));
-                double r = fma(-c1, a.q[i], x[i]);
+                a.w[i] = fma(c1, e.p2, fma(c0, e.p1, e.p0));
+                const double r = fma(-c1, e.p3, e.p4);
                 z[i] = r;
                 acc[0] = fma(r, r, acc[0]);
-                acc[1] = fma(a.y[i], r, acc[1]);
+                acc[ND - 1] = fma(a.y[i], r, acc[ND - 1]);
             } else if (mode == 1) {
-                a.w[i] = fma(c0, a.u[i], a.w[i]);
+                a.w[i] = fma(c0, e.p1, e.p0);
             }
         } else if (OP == V_CG_XR) {
             // w = x (solution), u = p, q = A p, z = r
             if (!mode) {
-                a.w[i] = fma(c0, a.u[i], a.w[i]);
-                const double r = fma(-c0, a.q[i], z[i]);
+                a.w[i] = fma(c0, e.p1, e.p0);
+                const double r = fma(-c0, e.p2, e.p3);
                 z[i] = r;
                 acc[0] = fma(r, r, acc[0]);
             }
         } else if (OP == V_CG_P) {
             // x = z (preconditioned residual), z = p
-            z[i] = mode ? x[i] : fma(c0, z[i], x[i]);
+            z[i] = mode ? e.p0 : fma(c0, e.p1, e.p0);
         } else if (OP == V_AXPY_ST1) {
-            z[i] += x[i];
+            z[i] = e.p1 + e.p0;
         } else if (OP == V_ZERO_IF_ST) {
             z[i] = 0.0;
         }
+    };
+    constexpr int kUnroll = OP == V_BICG_XR ? 2 : 4;
+    const int stride = gridDim.x * kThreads;
+    int i = blockIdx.x * kThreads + threadIdx.x;
+    for (; i < a.n - (kUnroll - 1) * stride; i += kUnroll * stride) {
+        Elem e[kUnroll];
+#pragma unroll
+        for (int q = 0; q < kUnroll; ++q)
+            e[q] = load(i + q * stride);
+#pragma unroll
+        for (int q = 0; q < kUnroll; ++q)
+            store(i + q * stride, e[q]);
     }
+    for (; i < a.n; i += stride)
+        store(i, load(i));
     if constexpr (ND > 0) {
         double v[ND];
 #pragma unroll
@@ -232,9 +277,37 @@ __device__ __forceinline__ float ld_basis(const float *p, uint64_t pol)
 
 constexpr int kGroup = 8; // basis vectors per CTA in a projection
 
+// Sums of kGroup per-thread values over a warp: the lane whose bits 4..2 are
+// q ends with the warp's sum of value (bit 4: value bit 2, bit 3: value bit
+// 1, bit 2: value bit 0).  Each halving step adds half as many values as the
+// one before, so a warp takes 4 + 2 + 1 + 1 + 1 = 9 FP64 adds for 8 values
+// where 8 separate shuffle sums take 40: on this part's FP64 pipe those sums
+// cost as much as the projection itself (n = 2,097,152, k = 30 in 4,864 CTAs).
+__device__ __forceinline__ double warp_sum_group(double (&v)[kGroup], int lane)
+{
+#pragma unroll
+    for (int h = kGroup / 2, o = 16; h >= 1; h >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int q = 0; q < h; ++q) {
+            const double keep = up ? v[q + h] : v[q];
+            const double send = up ? v[q] : v[q + h];
+            v[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    double t = v[0];
+    t += __shfl_xor_sync(0xffffffffu, t, 2);
+    t += __shfl_xor_sync(0xffffffffu, t, 1);
+    return t;
+}
+
 // h[i] = (V_i, w), i < k.  Grid (row blocks, vector groups); every CTA keeps
 // kGroup running sums per thread (in T) and reduces them once at the end (in
-// FP64, fixed order).
+// FP64, fixed order).  In FP64 the multiply-adds bound it: k n of them at two
+// per cycle and SM (2,097,152 x 30: 101 us at 2.07 GHz, the HBM stream 78),
+// so the grid holds only as many CTAs as run at once and each pays one
+// reduction for many rows, and two rows' loads are in flight per thread:
+// 166 -> 121 us (k = 8: 74 -> 43).
 template <class T> __global__ void __launch_bounds__(kThreads) k_multidot(BasisArgs a)
 {
     count_launch(a.st);
@@ -245,37 +318,55 @@ template <class T> __global__ void __launch_bounds__(kThreads) k_multidot(BasisA
         k = a.st->jend;
     const T *V = reinterpret_cast<const T *>(a.V);
     const T *w = reinterpret_cast<const T *>(a.w);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ double sh[kThreads / 32][kGroup];
+    __shared__ int s_last;
     const int g0 = blockIdx.y * kGroup;
-    T acc[kGroup];
-#pragma unroll
-    for (int q = 0; q < kGroup; ++q)
-        acc[q] = T(0);
     if (g0 < k) {
+        T acc[kGroup];
+#pragma unroll
+        for (int q = 0; q < kGroup; ++q)
+            acc[q] = T(0);
         const uint64_t pol = basis_policy();
         const int stride = gridDim.x * kThreads;
-        for (int i = blockIdx.x * kThreads + threadIdx.x; i < a.n; i += stride) {
+        const T *Vg = V + (int64_t)g0 * a.ldv;
+        const int cnt = min(kGroup, k - g0); // vectors of this group
+        int i = blockIdx.x * kThreads + threadIdx.x;
+        for (; i < a.n - stride; i += 2 * stride) { // two rows' loads in flight
+            T v0[kGroup], v1[kGroup];
+#pragma unroll
+            for (int q = 0; q < kGroup; ++q)
+                if (q < cnt) {
+                    v0[q] = ld_basis(&Vg[q * a.ldv + i], pol);
+                    v1[q] = ld_basis(&Vg[q * a.ldv + i + stride], pol);
+                }
+            const T w0 = w[i], w1 = w[i + stride];
+#pragma unroll
+            for (int q = 0; q < kGroup; ++q)
+                if (q < cnt)
+                    acc[q] = fma(v1[q], w1, fma(v0[q], w0, acc[q]));
+        }
+        if (i < a.n) {
             const T wi = w[i];
 #pragma unroll
             for (int q = 0; q < kGroup; ++q)
-                if (g0 + q < k)
-                    acc[q] = fma(ld_basis(&V[(int64_t)(g0 + q) * a.ldv + i], pol), wi, acc[q]);
+                if (q < cnt)
+                    acc[q] = fma(ld_basis(&Vg[q * a.ldv + i], pol), wi, acc[q]);
         }
-    }
-    // block reduction of the kGroup sums
-    __shared__ double sh[kGroup][kThreads / 32];
-    __shared__ int s_last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        double v[kGroup];
 #pragma unroll
-    for (int q = 0; q < kGroup; ++q) {
-        double t = warp_sum(double(acc[q]));
-        if (lane == 0)
-            sh[q][wid] = t;
+        for (int q = 0; q < kGroup; ++q)
+            v[q] = double(acc[q]);
+        const double t = warp_sum_group(v, lane);
+        if ((lane & 3) == 0)
+            sh[wid][(lane >> 2) & 7] = t; // lane bits 4..2 = value bits 2..0
     }
     __syncthreads();
-    if (threadIdx.x < kGroup) {
+    if (g0 < k && threadIdx.x < kGroup) {
         double t = 0.0;
+#pragma unroll
         for (int ww = 0; ww < kThreads / 32; ++ww)
-            t += sh[threadIdx.x][ww];
+            t += sh[ww][threadIdx.x];
         // partials layout: [vector][row block]
         const int q = g0 + threadIdx.x;
         if (q < k)
@@ -291,25 +382,42 @@ template <class T> __global__ void __launch_bounds__(kThreads) k_multidot(BasisA
     if (!s_last)
         return;
     __threadfence();
-    for (int q = threadIdx.x; q < k; q += kThreads) {
+    // the last CTA: eight lanes per vector, each over every eighth partial
+    for (int q0 = 0; q0 < k; q0 += kThreads / 8) {
+        const int q = q0 + threadIdx.x / 8, part = threadIdx.x % 8;
         double t = 0.0;
-        for (unsigned c = 0; c < gridDim.x; ++c)
-            t += __ldcg(&a.red.partials[(size_t)q * gridDim.x + c]);
-        if (a.op == FIN_GMRES_H1)
-            a.st->h1[q] = t;
-        else if (a.op == FIN_GMRES_H2)
-            a.st->h2[q] = t;
-        else
-            a.result[q] = t;
+        if (q < k) {
+            const double *pq = &a.red.partials[(size_t)q * gridDim.x];
+#pragma unroll 4
+            for (unsigned c = part; c < gridDim.x; c += 8)
+                t += __ldcg(&pq[c]);
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+            t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (q < k && part == 0) {
+            if (a.op == FIN_GMRES_H1)
+                a.st->h1[q] = t;
+            else if (a.op == FIN_GMRES_H2)
+                a.st->h2[q] = t;
+            else
+                a.result[q] = t;
+        }
     }
     if (threadIdx.x == 0)
         *a.red.ticket = 0u;
 }
 
-int launch_multidot(const BasisArgs &a, int grid, cudaStream_t s, bool fp32)
+int launch_multidot(const BasisArgs &a, int sms, cudaStream_t s, bool fp32)
 {
-    // a.k is the number of vectors, or an upper bound of it when k_from_st
-    dim3 g(grid, (a.k + kGroup - 1) / kGroup);
+    // a.k is the number of vectors, or an upper bound of it when k_from_st.
+    // Row blocks: FP64, at most kMultidotCtas CTAs per SM over all groups;
+    // FP32, two per SM and group -- more rows per thread would lengthen its
+    // FP32 running sums.
+    const int groups = (a.k + kGroup - 1) / kGroup;
+    const int cap = fp32 ? 2 * sms : max(1, sms * kMultidotCtas / groups);
+    const int need = (int)(((int64_t)a.n + kThreads - 1) / kThreads);
+    dim3 g(min(need, cap), groups);
     if (fp32)
         k_multidot<float><<<g, kThreads, 0, s>>>(a);
     else
@@ -338,7 +446,17 @@ template <bool NORM, class T> __global__ void __launch_bounds__(kThreads) k_basi
     const int stride = gridDim.x * kThreads;
     for (int i = blockIdx.x * kThreads + threadIdx.x; i < a.n; i += stride) {
         T t = w[i];
-        for (int q = 0; q < k; ++q)
+        int q = 0;
+        for (; q + kGroup <= k; q += kGroup) { // a group's loads first
+            T v[kGroup];
+#pragma unroll
+            for (int g = 0; g < kGroup; ++g)
+                v[g] = ld_basis(&V[(int64_t)(q + g) * a.ldv + i], pol);
+#pragma unroll
+            for (int g = 0; g < kGroup; ++g)
+                t = fma(-sc[q + g], v[g], t);
+        }
+        for (; q < k; ++q)
             t = fma(-sc[q], ld_basis(&V[(int64_t)q * a.ldv + i], pol), t);
         wout[i] = t;
         if (NORM)
@@ -385,7 +503,17 @@ template <class T> __global__ void __launch_bounds__(kThreads) k_basis_combine(B
     const int stride = gridDim.x * kThreads;
     for (int i = blockIdx.x * kThreads + threadIdx.x; i < a.n; i += stride) {
         T t = T(0);
-        for (int q = 0; q < k; ++q)
+        int q = 0;
+        for (; q + kGroup <= k; q += kGroup) { // a group's loads first
+            T v[kGroup];
+#pragma unroll
+            for (int g = 0; g < kGroup; ++g)
+                v[g] = ld_basis(&V[(int64_t)(q + g) * a.ldv + i], pol);
+#pragma unroll
+            for (int g = 0; g < kGroup; ++g)
+                t = fma(sc[q + g], v[g], t);
+        }
+        for (; q < k; ++q)
             t = fma(sc[q], ld_basis(&V[(int64_t)q * a.ldv + i], pol), t);
         wout[i] = t;
     }

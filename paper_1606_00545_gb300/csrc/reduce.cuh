@@ -171,43 +171,6 @@ __device__ inline void finalize(int op, const double *s, int nd, double *result,
     case FIN_GMRES_W0:
         st->w0norm = sqrt(s[0]);
         break;
-    case FIN_GMRES_STEP: {
-        const int j = st->j, m = st->restart;
-        const int ld = kMaxRestart;
-        double hn = sqrt(s[0]);
-        for (int i = 0; i <= j; ++i)
-            st->H[i * ld + j] = st->h1[i] + st->h2[i];
-        st->H[(j + 1) * ld + j] = hn;
-        for (int i = 0; i < j; ++i) {
-            double a = st->H[i * ld + j], c = st->H[(i + 1) * ld + j];
-            st->H[i * ld + j] = st->cs[i] * a + st->sn[i] * c;
-            st->H[(i + 1) * ld + j] = -st->sn[i] * a + st->cs[i] * c;
-        }
-        double a = st->H[j * ld + j], c = st->H[(j + 1) * ld + j];
-        double den = sqrt(a * a + c * c);
-        st->cs[j] = (den == 0.0) ? 1.0 : a / den;
-        st->sn[j] = (den == 0.0) ? 0.0 : c / den;
-        st->H[j * ld + j] = den;
-        st->H[(j + 1) * ld + j] = 0.0;
-        st->g[j + 1] = -st->sn[j] * st->g[j];
-        st->g[j] = st->cs[j] * st->g[j];
-        st->iters += 1;
-        double est = fabs(st->g[j + 1]);
-        st->est = est / st->bnorm;
-        int happy = (hn == 0.0) || (hn <= 1e-300 * st->w0norm);
-        int end = (est <= st->tol * st->bnorm) || happy || (j + 1 == m) ||
-                  (st->iters >= st->maxit) || isnan(est) ||
-                  (est <= st->inner_rtol * st->beta_cycle);
-        st->cycle_end = end;
-        if (end) {
-            st->jend = j + 1;
-        } else {
-            st->scale = 1.0 / hn;
-            st->j = j + 1;
-        }
-        set_cond(st, st->h_if, end);
-        break;
-    }
     case FIN_CG_INIT: {
         // r_0 = b - A x_0
         if (st->done)
@@ -275,6 +238,93 @@ __device__ inline void finalize(int op, const double *s, int nd, double *result,
     }
 }
 
+// FIN_GMRES_STEP: the Hessenberg column of step j, its Givens rotations and
+// the cycle tests.  All threads of the last CTA call it (s[0] = ||w''||^2 is
+// thread 0's): the column and the earlier rotations come into shared memory
+// with one load per thread, so the chain of rotations that thread 0 runs
+// (one dependent multiply-add per rotation) does not wait for memory.
+__device__ inline void finalize_gmres_step(const double *s, SolverState *st)
+{
+    __shared__ double hc[kMaxRestart], cs[kMaxRestart], sn[kMaxRestart];
+    const int j = st->j, m = st->restart;
+    const int ld = kMaxRestart;
+    for (int i = threadIdx.x; i <= j; i += kThreads) {
+        hc[i] = st->h1[i] + st->h2[i];
+        if (i < j) {
+            cs[i] = st->cs[i];
+            sn[i] = st->sn[i];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x != 0)
+        return;
+    const double hn = sqrt(s[0]);
+    double a = hc[0];
+    for (int i = 0; i < j; ++i) {
+        const double c = hc[i + 1];
+        st->H[i * ld + j] = cs[i] * a + sn[i] * c;
+        a = fma(-sn[i], a, cs[i] * c);
+    }
+    const double c = hn;
+    const double den = sqrt(a * a + c * c);
+    const double csj = (den == 0.0) ? 1.0 : a / den;
+    const double snj = (den == 0.0) ? 0.0 : c / den;
+    st->cs[j] = csj;
+    st->sn[j] = snj;
+    st->H[j * ld + j] = den;
+    st->H[(j + 1) * ld + j] = 0.0;
+    const double gj = st->g[j], gn = -snj * gj;
+    st->g[j + 1] = gn;
+    st->g[j] = csj * gj;
+    st->iters += 1;
+    const double est = fabs(gn);
+    st->est = est / st->bnorm;
+    int happy = (hn == 0.0) || (hn <= 1e-300 * st->w0norm);
+    int end = (est <= st->tol * st->bnorm) || happy || (j + 1 == m) ||
+              (st->iters >= st->maxit) || isnan(est) ||
+              (est <= st->inner_rtol * st->beta_cycle);
+    st->cycle_end = end;
+    if (end) {
+        st->jend = j + 1;
+    } else {
+        st->scale = 1.0 / hn;
+        st->j = j + 1;
+    }
+    set_cond(st, st->h_if, end);
+}
+
+// Sums of ND per-thread values over the CTA, in thread 0's s.  An FP64 add
+// of one warp holds its SM sub-partition's FP64 pipe for about 64 cycles
+// whatever the active lanes, so the sum is laid out for few warp-wide adds
+// and a short chain: the values go through shared memory, two warps per value
+// add four entries a lane (3 adds), reduce by shuffles (5), and thread 0 adds
+// the two (1).  17 warp-wide adds per value and CTA where shuffling in all 8
+// warps takes 48.  With grids of fewer CTAs (reduce_grid): a dot of 421,875
+// doubles 13.4 -> 8.3 us per call, of 2,097,152 14.5 -> 11.2 us.
+template <int ND> __device__ __forceinline__ void cta_sum(const double (&v)[ND], double (&s)[ND])
+{
+    static_assert(2 * ND <= kThreads / 32, "two warps per value");
+    __shared__ double sh[ND][kThreads];
+    __shared__ double half[ND][2];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int d = 0; d < ND; ++d)
+        sh[d][threadIdx.x] = v[d];
+    __syncthreads();
+    if (wid < 2 * ND) {
+        const double *p = &sh[wid >> 1][(wid & 1) * (kThreads / 2) + lane];
+        const double t = warp_sum((p[0] + p[32]) + (p[64] + p[96]));
+        if (lane == 0)
+            half[wid >> 1][wid & 1] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int d = 0; d < ND; ++d)
+            s[d] = half[d][0] + half[d][1];
+    }
+}
+
 // Block reduction of ND per-thread values, per-CTA partials, and a
 // fixed-order sum plus finalize() by the CTA that arrives last.  All threads
 // of the CTA must call it.  The summation order depends only on the grid
@@ -283,55 +333,39 @@ template <int ND>
 __device__ __forceinline__ void reduce_and_finalize(double (&v)[ND], const RedScratch &red, int op,
                                                     double *result, SolverState *st)
 {
-    __shared__ double sh[ND][kThreads / 32];
     __shared__ int s_last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int d = 0; d < ND; ++d) {
-        double t = warp_sum(v[d]);
-        if (lane == 0)
-            sh[d][wid] = t;
-    }
-    __syncthreads();
+    double s[ND];
+    cta_sum<ND>(v, s);
     const unsigned nblk = gridDim.x * gridDim.y;
     const unsigned bid = blockIdx.y * gridDim.x + blockIdx.x;
-    if (threadIdx.x == 0) {
+    if (nblk > 1) {
+        if (threadIdx.x == 0) {
+#pragma unroll
+            for (int d = 0; d < ND; ++d)
+                red.partials[(size_t)bid * ND + d] = s[d];
+            __threadfence();
+            unsigned tk = atomicAdd(red.ticket, 1u);
+            s_last = (tk == nblk - 1);
+        }
+        __syncthreads();
+        if (!s_last)
+            return;
+        __threadfence();
 #pragma unroll
         for (int d = 0; d < ND; ++d) {
             double t = 0.0;
-            for (int w = 0; w < kThreads / 32; ++w)
-                t += sh[d][w];
-            red.partials[(size_t)bid * ND + d] = t;
+            for (unsigned c = threadIdx.x; c < nblk; c += kThreads)
+                t += __ldcg(&red.partials[(size_t)c * ND + d]);
+            v[d] = t;
         }
-        __threadfence();
-        unsigned tk = atomicAdd(red.ticket, 1u);
-        s_last = (tk == nblk - 1);
+        cta_sum<ND>(v, s);
+        if (threadIdx.x == 0)
+            *red.ticket = 0u;
     }
-    __syncthreads();
-    if (!s_last)
-        return;
-    __threadfence();
-#pragma unroll
-    for (int d = 0; d < ND; ++d) {
-        double t = 0.0;
-        for (unsigned c = threadIdx.x; c < nblk; c += kThreads)
-            t += __ldcg(&red.partials[(size_t)c * ND + d]);
-        t = warp_sum(t);
-        if (lane == 0)
-            sh[d][wid] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s[ND];
-#pragma unroll
-        for (int d = 0; d < ND; ++d) {
-            s[d] = 0.0;
-            for (int w = 0; w < kThreads / 32; ++w)
-                s[d] += sh[d][w];
-        }
-        *red.ticket = 0u;
+    if (op == FIN_GMRES_STEP)
+        finalize_gmres_step(s, st);
+    else if (threadIdx.x == 0)
         finalize(op, s, ND, result, st);
-    }
 }
 
 } // namespace hec
