@@ -305,7 +305,7 @@ int reduce_grid(int64_t n)
 int run_vec(VecOp op, const VecArgs &a, cudaStream_t s)
 {
     const bool reduces = op == V_DOT || op == V_NRM2SQ || op == V_BICG_S || op == V_BICG_XR ||
-                         op == V_CG_XR;
+                         op == V_CG_XR || op == V_CG_XRZ;
     if (launch_vec(op, a, reduces ? reduce_grid(a.n) : vec_grid(a.n), s) != 0)
         return fail(HEC_ERR_INVALID, "bad vector op");
     return check_launch("vector op");
@@ -785,8 +785,23 @@ int seq_cg_body(hec_matrix_s *A, hec_precond_s *M, Solver &S, cudaStream_t cs)
     xr.q = S.q;
     xr.z = S.r;
     xr.op = FIN_CG_R;
-    HEC_TRY(run_vec(V_CG_XR, xr, cs)); // x, r updates, ||r||
-    return seq_cg_rz_p(M, S, cs);
+    if (M && M->kind != kJacobi) {
+        HEC_TRY(run_vec(V_CG_XR, xr, cs)); // x, r updates, ||r||
+        return seq_cg_rz_p(M, S, cs);
+    }
+    // z = d .* r (damped Jacobi, or d = 1) is formed where it is used: (r, z)
+    // with the updates and p = z + beta p, so a pass is three launches and
+    // z never goes through memory (75^3: 36 us a pass, 47 as five launches)
+    xr.v = M ? M->dinv.as<double>() : nullptr;
+    xr.op = FIN_CG_R_RHO;
+    HEC_TRY(run_vec(V_CG_XRZ, xr, cs)); // x, r updates, ||r||, (r, z), loop condition
+    VecArgs pz{};
+    pz.n = S.n;
+    pz.st = S.st;
+    pz.x = S.r;
+    pz.v = xr.v;
+    pz.z = S.p;
+    return run_vec(V_CG_PZ, pz, cs); // p = z + beta p
 }
 
 // Exit: x = 0 if b = 0; the true residual ||b - A x|| / ||b||.

@@ -11,11 +11,11 @@ __global__ void __launch_bounds__(kThreads) k_vec(VecArgs a)
     count_launch(a.st);
     SolverState *st = a.st;
     constexpr int ND = (OP == V_DOT || OP == V_NRM2SQ || OP == V_BICG_S || OP == V_CG_XR) ? 1
-                       : (OP == V_BICG_XR)                                                  ? 2
+                       : (OP == V_BICG_XR || OP == V_CG_XRZ)                                ? 2
                                                                                             : 0;
     if (OP == V_BICG_S && st->skip)
         return;
-    if (OP == V_CG_P && st->done)
+    if ((OP == V_CG_P || OP == V_CG_PZ) && st->done)
         return;
     if (OP == V_ZERO_IF_ST && !st->zero_x)
         return;
@@ -47,11 +47,11 @@ __global__ void __launch_bounds__(kThreads) k_vec(VecArgs a)
     }
     if (OP == V_BICG_S)
         c0 = st->alpha;
-    if (OP == V_CG_XR) {
+    if (OP == V_CG_XR || OP == V_CG_XRZ) {
         c0 = st->alpha;
         mode = st->skip; // breakdown in alpha: no update (the sum still runs)
     }
-    if (OP == V_CG_P) {
+    if (OP == V_CG_P || OP == V_CG_PZ) {
         mode = st->iters == 0; // first pass: p = z
         c0 = st->cg_beta;
     }
@@ -88,8 +88,13 @@ __global__ void __launch_bounds__(kThreads) k_vec(VecArgs a)
         } else if (OP == V_CG_XR) {
             if (!mode)
                 e = {a.w[i], a.u[i], a.q[i], z[i], 0};
-        } else if (OP == V_CG_P) {
+        } else if (OP == V_CG_XRZ) {
+            if (!mode)
+                e = {a.w[i], a.u[i], a.q[i], z[i], a.v ? a.v[i] : 1.0};
+        } else if (OP == V_CG_P || OP == V_CG_PZ) {
             e.p0 = x[i];
+            if (OP == V_CG_PZ && a.v)
+                e.p0 *= a.v[i];
             if (!mode)
                 e.p1 = z[i];
         } else if (OP == V_AXPY_ST1)
@@ -134,8 +139,17 @@ __global__ void __launch_bounds__(kThreads) k_vec(VecArgs a)
                 z[i] = r;
                 acc[0] = fma(r, r, acc[0]);
             }
-        } else if (OP == V_CG_P) {
-            // x = z (preconditioned residual), z = p
+        } else if (OP == V_CG_XRZ) {
+            // as V_CG_XR; v = d (null: ones), (r, d .* r) in the same pass
+            if (!mode) {
+                a.w[i] = fma(c0, e.p1, e.p0);
+                const double r = fma(-c0, e.p2, e.p3);
+                z[i] = r;
+                acc[0] = fma(r, r, acc[0]);
+                acc[ND - 1] = fma(r, __dmul_rn(e.p4, r), acc[ND - 1]);
+            }
+        } else if (OP == V_CG_P || OP == V_CG_PZ) {
+            // x = z (preconditioned residual; V_CG_PZ: r, scaled by v), z = p
             z[i] = mode ? e.p0 : fma(c0, e.p1, e.p0);
         } else if (OP == V_AXPY_ST1) {
             z[i] = e.p1 + e.p0;
@@ -186,6 +200,8 @@ int launch_vec(VecOp vop, const VecArgs &a, int grid, cudaStream_t s)
         HEC_VEC_CASE(V_ZERO_IF_ST)
         HEC_VEC_CASE(V_CG_XR)
         HEC_VEC_CASE(V_CG_P)
+        HEC_VEC_CASE(V_CG_XRZ)
+        HEC_VEC_CASE(V_CG_PZ)
 #undef HEC_VEC_CASE
     }
     return -1;

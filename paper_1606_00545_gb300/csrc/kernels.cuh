@@ -34,6 +34,7 @@ enum FinOp : int {
     FIN_CG_RHO,           // (r, z): rho, beta = rho_new / rho; loop condition
     FIN_CG_ALPHA,         // q = A p: alpha = rho / (p, q)
     FIN_CG_R,             // x, r update: ||r|| test, iteration count
+    FIN_CG_R_RHO,         // FIN_CG_R on sum 0, then FIN_CG_RHO on sum 1
 };
 
 // Device-resident solver state: scalars of Algorithm 4 / GMRES, loop flags,
@@ -108,6 +109,8 @@ enum VecOp : int {
     V_ZERO_IF_ST,  // z = 0 if st->zero_x
     V_CG_XR,       // x += alpha p, r -= alpha q, (r, r)          (CG)
     V_CG_P,        // p = z + beta p (first pass: p = z)           (CG)
+    V_CG_XRZ,      // V_CG_XR and (r, d .* r) in one pass      (CG, Jacobi or none)
+    V_CG_PZ,       // p = d .* r + beta p                       (CG, Jacobi or none)
     V_JACOBI,      // z = d .* x (typed: damped Jacobi, d = omega / a_ii)
 };
 struct VecArgs {

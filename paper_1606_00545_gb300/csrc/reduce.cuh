@@ -30,6 +30,44 @@ __device__ __forceinline__ void set_cond(const SolverState *st, cudaGraphConditi
         cudaGraphSetConditional(h, on ? 1u : 0u);
 }
 
+// (r_{j+1}, z_{j+1}): beta_j and the next rho; the loop goes on unless the
+// residual test, the budget or a breakdown ended it.
+__device__ inline void finalize_cg_rho(double rz, SolverState *st)
+{
+    if (!st->done) {
+        if (rz == 0.0 || isnan(rz)) {
+            st->done = 1;
+            st->status = HEC_BREAKDOWN;
+        } else {
+            st->cg_beta = (st->iters > 0) ? rz / st->rho : 0.0;
+            st->rho = rz;
+        }
+    }
+    st->skip = 0; // the last pass skipped its preconditioner apply; the exit runs
+    set_cond(st, st->h_while, !st->done);
+}
+
+// CG after the x, r update: ||r||^2, the residual test and the pass count.
+__device__ inline void finalize_cg_r(double rr, SolverState *st)
+{
+    if (st->skip)
+        return;
+    st->iters += 1;
+    const double rn = sqrt(rr);
+    st->est = rn / st->bnorm;
+    if (rn <= st->tol * st->bnorm) {
+        st->done = 1;
+        st->status = HEC_OK;
+    } else if (isnan(rn)) {
+        st->done = 1;
+        st->status = HEC_BREAKDOWN;
+    } else if (st->iters >= st->maxit) {
+        st->done = 1;
+        st->status = HEC_MAXIT;
+    }
+    st->skip = st->done; // no preconditioner apply after the last pass
+}
+
 // Scalar recurrences (one thread).  s[0..nd) are the reduced values.
 __device__ inline void finalize(int op, const double *s, int nd, double *result, SolverState *st)
 {
@@ -186,23 +224,9 @@ __device__ inline void finalize(int op, const double *s, int nd, double *result,
         }
         break;
     }
-    case FIN_CG_RHO: {
-        // (r_{j+1}, z_{j+1}): beta_j and the next rho; the loop goes on
-        // unless the residual test, the budget or a breakdown ended it
-        if (!st->done) {
-            const double rz = s[0];
-            if (rz == 0.0 || isnan(rz)) {
-                st->done = 1;
-                st->status = HEC_BREAKDOWN;
-            } else {
-                st->cg_beta = (st->iters > 0) ? rz / st->rho : 0.0;
-                st->rho = rz;
-            }
-        }
-        st->skip = 0; // the last pass skipped its preconditioner apply; the exit runs
-        set_cond(st, st->h_while, !st->done);
+    case FIN_CG_RHO:
+        finalize_cg_rho(s[0], st);
         break;
-    }
     case FIN_CG_ALPHA: {
         const double pq = s[0];
         if (pq == 0.0 || isnan(pq)) {
@@ -214,25 +238,13 @@ __device__ inline void finalize(int op, const double *s, int nd, double *result,
         }
         break;
     }
-    case FIN_CG_R: {
-        if (st->skip)
-            break;
-        st->iters += 1;
-        const double rn = sqrt(s[0]);
-        st->est = rn / st->bnorm;
-        if (rn <= st->tol * st->bnorm) {
-            st->done = 1;
-            st->status = HEC_OK;
-        } else if (isnan(rn)) {
-            st->done = 1;
-            st->status = HEC_BREAKDOWN;
-        } else if (st->iters >= st->maxit) {
-            st->done = 1;
-            st->status = HEC_MAXIT;
-        }
-        st->skip = st->done; // no preconditioner apply after the last pass
+    case FIN_CG_R:
+        finalize_cg_r(s[0], st);
         break;
-    }
+    case FIN_CG_R_RHO:
+        finalize_cg_r(s[0], st);
+        finalize_cg_rho(s[nd - 1], st);
+        break;
     default:
         break;
     }
