@@ -436,6 +436,7 @@ int pack_layout(const hec_precond_s *M, int idx, TrsvPack &P, int &fixed_width, 
     // ahead (the padding costs multiply-adds only where a warp's rows are
     // shorter than the width)
     fixed_width = trsv_uniform_width(longest);
+    P = TrsvPack(); // (a resident layout that did not fit leaves nothing behind)
     return pack_trsv(M->blocks, M->n, M->stage_bytes, kMaxRing, vb, P, msg, fixed_width,
                      layout_parts(M, idx));
 }

@@ -798,3 +798,15 @@ def test_spmv_rejects_misaligned_output(H):
     # aligned: rejected for the host-only handle instead, after the alignment check
     rc = lib.hec_spmv(M.handle, 1.0, x, 0.0, None, ctypes.c_void_p(0x20010), None, None, None)
     assert rc == H.ERR_INVALID and b"host-only" in lib.hec_last_error()
+
+
+def test_block_too_large_for_the_resident_kernel_streams(H):
+    """A block whose levels are narrow enough for the resident kernel but whose
+    vector does not fit in shared memory (30,000 FP64 rows) takes the streamed
+    layout, and the handle says so."""
+    A = synth.diffusion2d_5pt_lognormal(100, 1.0, 3, Ny=300)
+    M = H.hec_build(A.row_ptr, A.col, A.val, host_only=True)
+    P = H.ilu_k_setup(M, 0, 1, 0)
+    H.level_schedule(P)
+    assert P.info()["trsv_resident"] == 0
+    assert P.layout()["fixed_width"] == 4
