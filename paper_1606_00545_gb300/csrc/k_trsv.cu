@@ -22,7 +22,7 @@
 //   - an issuer warp streams chunks into a ring of shared-memory stages with
 //     cp.async.bulk (the TMA bulk-copy engine, evict-first in L2) completing
 //     on mbarriers, S chunks ahead of the solving warps;
-//   - two gatherer warps, taking chunks in turn, gather each landed chunk's
+//   - four gatherer warps, taking chunks in turn, gather each landed chunk's
 //     right-hand sides (L pass: from r; U pass: from the L results, once the
 //     L pass is complete) with 4- or 8-byte cp.async, one chunk ahead, and
 //     hand the chunk over (a per-stage release-add counter) once the copies
@@ -59,10 +59,13 @@ size_t trsv_smem_bytes(int stage_bytes, int nstages, int ring_slots, int vbytes)
            (size_t)(2 * nstages + 1) * sizeof(uint64_t) + 2 * sizeof(uint32_t);
 }
 
-// Gatherer warps of a CTA: each takes every other chunk and keeps two
-// chunks' right-hand-side gathers in flight.  (Three and four gatherers
-// were measured on the 128^3 case: no faster.)
-constexpr int kGatherers = 2;
+// Gatherer warps of a CTA: they take the chunks in turn and keep up to
+// kGatherDepth chunks' right-hand-side gathers in flight each.  (Two, three
+// or four gatherers, depths 2 and 4: within 4% on the 128^3 case.)
+constexpr int kGatherers = 4;
+constexpr int kGatherDepth = 2;
+
+constexpr int kMaxStages = 16; // of the streamed kernel
 
 int trsv_stages_for(int stage_bytes, int ring_slots, int vbytes)
 {
@@ -70,7 +73,8 @@ int trsv_stages_for(int stage_bytes, int ring_slots, int vbytes)
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         optin = 227 * 1024;
-    int S = 8;
+    optin -= 1024; // static shared memory of the kernel
+    int S = kMaxStages;
     while (S > 3 && trsv_smem_bytes(stage_bytes, S, ring_slots, vbytes) > (size_t)optin)
         --S;
     return S;
@@ -123,7 +127,6 @@ constexpr long long kDrainPolls = 1ll << 24;
 constexpr int kWarpRows = 32;
 constexpr int kMaxWarps = kThreads / kWarpRows;
 constexpr int kFeedThreads = 32 * (kGatherers + 2); // issuer, gatherers and the signaller
-constexpr int kMaxStages = 8;
 
 __device__ __forceinline__ int seg_stride(int w, int nrows)
 {
@@ -242,8 +245,8 @@ __device__ __forceinline__ T row_solve_any(const Segment<T> &g, int lane, const 
     }
 }
 
-// Barrier of the consumer warps only (named barrier 1), AND-reducing a flag.
-__device__ __forceinline__ int consumer_sync_and(int flag)
+// Barrier of the NT solving threads only (named barrier 1), AND-reducing a flag.
+template <int NT> __device__ __forceinline__ int solvers_sync_and(int flag)
 {
     int all;
     asm volatile("{\n\t.reg .pred p, q;\n\t"
@@ -251,9 +254,27 @@ __device__ __forceinline__ int consumer_sync_and(int flag)
                  "barrier.cta.red.and.pred q, 1, %2, p;\n\t"
                  "selp.s32 %0, 1, 0, q;\n\t}"
                  : "=r"(all)
-                 : "r"(flag), "n"(kThreads)
+                 : "r"(flag), "n"(NT)
                  : "memory");
     return all;
+}
+
+#ifdef HEC_DEBUG
+// Barrier of one set of solving warps (named barriers 2 and 3).
+__device__ __forceinline__ void solvers_set_sync(int set)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + set), "n"(kThreads) : "memory");
+}
+#endif
+
+// Plain barrier of the NT solving threads (named barrier 1).  Measured on
+// GB300: 19 cycles for 4 warps, the AND-reducing form 60; so the two-set loops
+// use this one.  They do not leave early on a failed wait: it sets a shared
+// word, and from then on a set loads nothing more, so the remaining levels
+// are barriers only.
+template <int NT> __device__ __forceinline__ void solvers_sync()
+{
+    asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
 }
 
 // ------------------------------------------------------------------ generic format
@@ -324,12 +345,13 @@ template <class T, int FW> struct RowRegs {
     __device__ int d(int k) const { return get4(dv[k / 4], k % 4); }
 };
 
-// Every address below depends only on the stage, the thread and the pass,
-// never on a value read from the stage: all loads issue back to back, 16
-// bytes each for the row's entries.
+// Row t = 32 w + lane of a chunk.  Warps past the chunk's last one read the
+// header only; past it, every address depends on the stage, the thread and
+// the pass alone: all loads issue back to back, 16 bytes each for the row's
+// entries.
 template <class T, int FW>
 __device__ __forceinline__ void load_fixed(const unsigned char *ch, const T *rslot, int w, int lane,
-                                           int t, bool upass, bool exps, RowRegs<T, FW> &R)
+                                           bool upass, bool exps, RowRegs<T, FW> &R)
 {
     using F = Fixed<T, FW>;
     const int4 hdr = *reinterpret_cast<const int4 *>(ch);
@@ -337,6 +359,8 @@ __device__ __forceinline__ void load_fixed(const unsigned char *ch, const T *rsl
     R.nwarps = hdr.y;
     R.base = hdr.z;
     R.flags = hdr.w;
+    if (w >= hdr.y)
+        return;
     const unsigned char *blk = ch + kFixedHeader + (size_t)w * F::block(upass, exps);
     const typename Vec16<T>::type *val = reinterpret_cast<const typename Vec16<T>::type *>(blk) + lane;
 #pragma unroll
@@ -346,7 +370,7 @@ __device__ __forceinline__ void load_fixed(const unsigned char *ch, const T *rsl
 #pragma unroll
     for (int v = 0; v < F::ND; ++v)
         R.dv[v] = dep[v * 32];
-    R.rhs = rslot[t];
+    R.rhs = rslot[w * kWarpRows + lane];
     if (upass) {
         R.dinv = reinterpret_cast<const T *>(blk + F::dinv())[lane];
         R.dst = reinterpret_cast<const int *>(blk + F::dst(true))[lane];
@@ -396,45 +420,50 @@ __device__ __forceinline__ bool issue_chunks(const uint2 *chunks, int nch, int S
     return true;
 }
 
-// Release-add by one thread to a shared counter (the handover of a chunk).
-__device__ __forceinline__ void red_release_add(uint32_t *p, uint32_t v)
-{
-    asm volatile("red.release.cta.shared::cta.add.u32 [%0], %1;" ::"r"(smem_u32(p)), "r"(v)
-                 : "memory");
-}
-
-// Warp-specialised CTA: warps 0-7 solve rows (one row per thread per chunk),
-// warps 8-11 feed them.  Per chunk c in stage s = c mod S:
-//   issuer (warp 8): wait empty[s] (chunk c - S released) -> arm full[s] with
+// Warp-specialised CTA: 8 warps (fixed-slot chunks: two sets of 8) solve rows,
+// one row per thread per chunk; the last six warps feed them.  Per chunk c
+// in stage s = c mod S:
+//   issuer: wait empty[s] (chunk c - S released) -> arm full[s] with
 //             the chunk's byte count -> cp.async.bulk the chunk;
-//   gatherers (warps 9 and 10, chunks alternating): wait full[s] -> gather
+//   gatherers (four warps, chunks in turn): wait full[s] -> gather
 //             the chunk's right-hand sides into slot s with cp.async, one
 //             commit group per chunk (a U chunk waits for ldone first: its
 //             right-hand side is the L pass's output) -> once the group has
-//             completed (waited for while the warp's next chunk is gathered)
+//             completed (waited for while the warp's next chunks are gathered)
 //             and lane 0 has seen the neighbouring parts' progress counters
-//             reach the chunk's thresholds, every lane adds 1 to the stage's
-//             handover counter (release): 32 per chunk;
-//   consumers: fixed-slot chunks are software-pipelined by one chunk: after
-//             issuing chunk c's dependency loads, every thread copies its row
-//             of chunk c + 1 into registers, then runs chunk c's multiply-add
-//             chain.  The level's results go to the ring (and, for exports,
-//             into the neighbour's import ring).  Before the level's barrier
-//             the last thread -- whose warp holds the shortest rows --
-//             confirms that chunk c + 2 has been handed over (an acquire load
-//             of the counter; the barrier orders everybody's later loads
-//             after it), and after the barrier it frees chunk c + 1's stage
-//             and publishes the completed count.  Generic chunks are solved
-//             from shared memory, one at a time;
-//   signaller (warp 11): for a split block, forwards the completed count to
+//             reach the chunk's thresholds, lane 0 arrives on the stage's
+//             handover mbarrier (a release-add to a shared counter instead
+//             waits for every copy of the warp still in flight);
+//   solvers, fixed-slot chunks: two sets of 8 warps take the chunks in turn,
+//             and a barrier of both ends every level.  While one set solves
+//             chunk c -- ring loads, the row's multiply-add chain, the result
+//             into the ring (for exports also into the neighbour's import
+//             ring) -- the other confirms that chunk c + 1 has been handed
+//             over, copies its rows into registers and forms every address
+//             its level will need.  So a level's critical path holds none of
+//             that: with one set doing all of it, the next chunk's copy and
+//             address arithmetic were the longer half of a level.  128^3,
+//             ILU(1), 64 blocks in two parts: FP64 apply 428 -> 330 us;
+//             101^3: 557 -> 463; 32^3, 8 blocks: 109 -> 78 (FP32 72 -> 52).
+//             Three sets of 4 warps, with the addresses formed in a level of
+//             their own, were no faster (335 us), and adding the older
+//             levels' entries ahead of the barrier slower (410): the FP64
+//             unit is shared by the SM (16 cycles a warp-wide multiply-add,
+//             one in flight per warp), so the two sets then queue for it;
+//   solvers, generic chunks: one set, rows solved from shared memory;
+//   signaller: for a split block, forwards the completed count to
 //             the neighbouring parts (a release at cluster scope, then the
 //             count stored into their shared memory) as often as the fence
 //             allows -- the count may jump several chunks at once.
 // T = double: the FP64 path; T = float: the FP32 inner solves of the
 // mixed-precision mode (FP32 factors, products and accumulation).
+// Solving threads of a CTA: two sets of 8 warps for fixed-slot chunks.
+template <int FW> constexpr int kSolvers = FW > 0 ? 2 * kThreads : kThreads;
+
 template <class T, int FW>
-__global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArgs a)
+__global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(TrsvArgs a)
 {
+    constexpr int NT = kSolvers<FW>; // solving threads; the feeding warps follow
     extern __shared__ __align__(128) unsigned char smem[];
     count_launch(a.st);
     if (a.st && a.st->skip)
@@ -474,12 +503,13 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
     // shared state of the roles (written before the final barrier)
     __shared__ int s_issued, s_err;
     __shared__ uint32_t s_done;             // chunks the consumers have completed
-    __shared__ uint32_t s_hand[kMaxStages]; // handover count of every stage: 32 per chunk
+    __shared__ uint64_t s_hand[kMaxStages]; // handover mbarrier of every stage: a phase per chunk
 
     if (t == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
+            mbar_init(&s_hand[s], 1);
         }
         mbar_init(ldone, 1);
         ctr[0] = ctr[1] = 0;
@@ -488,8 +518,6 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
         s_done = 0;
         fence_mbar_init();
     }
-    if (t < kMaxStages)
-        s_hand[t] = 0;
     for (int i = t; i < nown; i += blockDim.x)
         ring[i] = T(0);
     __syncthreads();
@@ -499,94 +527,112 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
         cluster_sync_all();
     int failed = 0;
 
-    if (t >= kThreads && t < kThreads + 32 && !stall_test) {
+    if (t >= NT && t < NT + 32 && !stall_test) {
         // ------------------------------------------------------------ issuer warp
         if (!issue_chunks(chunks, nch, S, a.stage_bytes, a.pack, stages, full, empty, limit,
-                          t - kThreads, &s_issued))
+                          t - NT, &s_issued))
             failed = 1;
-    } else if (t >= kThreads + 32 && t < kThreads + 32 * (1 + kGatherers) && !stall_test) {
+    } else if (t >= NT + 32 && t < NT + 32 * (1 + kGatherers) && !stall_test) {
         // ------------------------------------------------------------ gatherer warps
-        // follow the chunks as they land (even chunks: warp 9, odd: warp 10):
+        // follow the chunks as they land, in turn:
         // gather each one's right-hand sides as one cp.async group, and hand
         // the chunk over once its group has completed and the neighbours'
-        // progress allows it.  Each warp keeps one chunk's gathers in flight
-        // while it issues the next one's.  Every lane hands over for itself,
-        // after waiting for its own copies (an arrive-on-completion of the
+        // progress allows it.  Every lane waits for its own copies before the
+        // warp's vote and lane 0's release (an arrive-on-completion of the
         // copies, measured on this GPU, did not make them visible to the
         // solving warps in time).
-        const int gw = (t - kThreads - 32) / 32;
+        const int gw = (t - NT - 32) / 32;
         const int lane = t % 32;
         bool ldone_seen = false;
-        int sg = gw; // S >= 3: chunk gw lies in stage gw, phase 0
+        // with 3 or 4 stages two of them work: the phase tests below tell a
+        // stage's uses apart when a chunk that this warp saw land was issued
+        // after the stage's last use but one was released (S >= NG)
+        const int NG = S > kGatherers ? kGatherers : 2;
+        int sg = gw; // gw < NG <= S: chunk gw lies in stage gw, phase 0
         uint32_t par = 0;
-        int gp = -1, sgp = 0; // the chunk whose gathers are in flight, and its stage
-        // hand chunk gp over: lane 0 first waits for the neighbours' progress
+        int seen0 = 0, seen1 = 0; // lane 0: the neighbours' progress seen last
+        int sh = sg, pend = 0; // stage of the oldest chunk in flight; chunks in flight
+        // hand the oldest chunk over: its copies have landed, and lane 0 waits
+        // for the neighbours' progress
         auto finish = [&]() -> bool {
+            switch (pend) { // groups committed after it (kGatherDepth = 2)
+            case 1: cp_async_wait_group<0>(); break;
+            default: cp_async_wait_group<kGatherDepth - 1>(); break;
+            }
             int late = 0;
             if (lane == 0 && clustered) {
                 // the values this chunk imports are in the ring, and the
                 // import slots its exports overwrite have been read
-                const unsigned char *ch = stages + (size_t)sgp * a.stage_bytes;
+                const unsigned char *ch = stages + (size_t)sh * a.stage_bytes;
                 const int2 need = *reinterpret_cast<const int2 *>(ch + (FW > 0 ? 16 : 96));
                 long long it = 0;
-                // polls back off, leaving the issue slots to the solving warps
-                if (need.x > 0)
-                    while ((int)ld_acquire_cluster_u32(&ctr[0]) < need.x && ++it < limit)
-                        __nanosleep(32);
-                if (need.y > 0)
-                    while ((int)ld_acquire_cluster_u32(&ctr[1]) < need.y && ++it < limit)
-                        __nanosleep(32);
+                // polls back off, leaving the issue slots to the solving warps;
+                // none where the progress seen last covers the chunk
+                while (seen0 < need.x && (seen0 = (int)ld_acquire_cluster_u32(&ctr[0])) < need.x &&
+                       ++it < limit)
+                    __nanosleep(32);
+                while (seen1 < need.y && (seen1 = (int)ld_acquire_cluster_u32(&ctr[1])) < need.y &&
+                       ++it < limit)
+                    __nanosleep(32);
                 late = it >= limit;
             }
+            // (the vote also orders every lane's landed copies before the release)
             if (__any_sync(0xffffffffu, late))
                 return false;
-            red_release_add(&s_hand[sgp], 1u); // this lane's gathers of chunk gp have landed
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(&s_hand[sh]);
+            sh += NG;
+            if (sh >= S)
+                sh -= S;
+            --pend;
             return true;
         };
-        for (int g = gw; g < nch; g += kGatherers) {
-            // a chunk in flight is handed over first when the next one has not landed
-            if (gp >= 0 && !__all_sync(0xffffffffu, mbar_test_wait(&full[sg], par))) {
-                cp_async_wait_group<0>();
+        for (int g = gw; gw < NG && g < nch;) {
+            // chunks in flight are handed over first when the next one has not
+            // landed, or needs the whole L pass
+            const bool wait_l = g >= nL && !ldone_seen;
+            // (the stage's previous chunk has been released, then its next landed)
+            if (pend > 0 &&
+                (pend == kGatherDepth || wait_l ||
+                 !__all_sync(0xffffffffu, (g < S || mbar_test_wait(&empty[sg], par ^ 1u)) &&
+                                              mbar_test_wait(&full[sg], par)))) {
                 if (!finish()) {
                     failed = 1;
                     break;
                 }
-                gp = -1;
+                continue;
             }
-            if (__any_sync(0xffffffffu, !bounded_wait(&full[sg], par, limit))) {
+            if ((g >= S && __any_sync(0xffffffffu, !bounded_wait(&empty[sg], par ^ 1u, limit))) ||
+                __any_sync(0xffffffffu, !bounded_wait(&full[sg], par, limit)) ||
+                (wait_l && __any_sync(0xffffffffu, !bounded_wait(ldone, 0u, limit)))) {
                 failed = 1;
                 break;
             }
+            ldone_seen |= wait_l;
             const unsigned char *ch = stages + (size_t)sg * a.stage_bytes;
             int4 hdr = *reinterpret_cast<const int4 *>(ch);
             const bool upass = (hdr.w & 1) != 0;
             if (!HEC_CHECK(upass == (g >= nL), 1, g, hdr.w, nL) ||
                 !HEC_CHECK(hdr.x >= 1 && hdr.x <= kThreads, 2, g, hdr.x, kThreads))
                 hdr.x = 0; // nothing gathered from a chunk that is not the expected one
-            if (upass && !ldone_seen) {
-                if (gp >= 0) { // the last L chunk in flight goes first
-                    cp_async_wait_group<0>();
-                    if (!finish()) {
-                        failed = 1;
-                        break;
-                    }
-                    gp = -1;
-                }
-                if (__any_sync(0xffffffffu, !bounded_wait(ldone, 0u, limit))) {
-                    failed = 1;
-                    break;
-                }
-                ldone_seen = true;
-            }
             T *slot = rhs + (size_t)sg * kThreads;
             const T *from = upass ? ysc : r;
             if constexpr (FW > 0) {
                 const int blkb = Fixed<T, FW>::block(upass, exps);
                 const unsigned char *src = ch + kFixedHeader + Fixed<T, FW>::src(upass) + 4 * lane;
-                for (int i = lane, j = 0; i < hdr.x; i += 32, ++j) {
-                    const int si = *reinterpret_cast<const int *>(src + (size_t)j * blkb);
-                    if (HEC_CHECK(si >= 0 && (upass || si < a.n), 3, g, si, a.n))
-                        cp_async_v<sizeof(T)>(&slot[i], from + si);
+                for (int i0 = 0; i0 < hdr.x; i0 += 128) { // four rows' sources read at once
+                    int si[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (i0 + 32 * q + lane < hdr.x)
+                            si[q] = *reinterpret_cast<const int *>(
+                                src + (size_t)(i0 / 32 + q) * blkb);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (i0 + 32 * q + lane < hdr.x &&
+                            HEC_CHECK(si[q] >= 0 && (upass || si[q] < a.n), 3, g, si[q], a.n))
+                            cp_async_v<sizeof(T)>(&slot[i0 + 32 * q + lane], from + si[q]);
                 }
             } else {
                 const ChunkView<T> v = view_chunk<T>(ch);
@@ -595,33 +641,24 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
                         cp_async_v<sizeof(T)>(&slot[i], from + v.src[i]);
             }
             cp_async_commit();
-            if (gp >= 0) { // the previous chunk's group: all but the newest have completed
-                cp_async_wait_group<1>();
-                if (!finish()) {
-                    failed = 1;
-                    break;
-                }
-            }
-            gp = g;
-            sgp = sg;
-            sg += kGatherers;
+            ++pend;
+            g += NG;
+            sg += NG;
             if (sg >= S) {
                 sg -= S;
                 par ^= 1u;
             }
         }
-        if (!failed && gp >= 0) {
-            cp_async_wait_group<0>();
+        while (!failed && pend > 0)
             if (!finish())
                 failed = 1;
-        }
         cp_async_wait_all();
-    } else if (t >= kThreads + 32 * (1 + kGatherers)) {
+    } else if (t >= NT + 32 * (1 + kGatherers)) {
         // ------------------------------------------------------------ signaller warp
         // publishes the completed-chunk count to the neighbours: the release
         // at cluster scope covers the consumers' stores into the neighbours'
         // import rings, ordered before the count by the consumer barrier
-        if (signal && t == kThreads + 32 * (1 + kGatherers)) {
+        if (signal && t == NT + 32 * (1 + kGatherers)) {
             const uint32_t to_prev = has_prev ? mapa_shared(smem_u32(&ctr[1]), part - 1) : 0;
             const uint32_t to_next = has_next ? mapa_shared(smem_u32(&ctr[0]), part + 1) : 0;
             uint32_t pub = 0;
@@ -644,7 +681,7 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
                 }
             }
         }
-    } else if (t < kThreads) {
+    } else if (t < NT) {
     // ---------------------------------------------------------------- consumer warps
     volatile int *verr = &s_err;
     // the neighbours' import rings: L values go to part p + 1, U values to p - 1
@@ -653,18 +690,10 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
     const uint32_t imp_prev =
         has_prev ? mapa_shared(smem_u32(ring + nown), part - 1) : 0;
     int s = 0;         // stage of chunk c
-    uint32_t hneed = 32; // the stage's handover count once chunk c is handed over
+    uint32_t hpar = 0; // the parity of that stage's handover of chunk c
     int err = 0;
-    // wait (bounded) until chunk c, in stage s, has been handed over
-    auto handed = [&](int st, uint32_t need) -> bool {
-        long long it = 0;
-        while (ld_acquire_cta_u32(&s_hand[st]) < need) {
-            if (++it >= limit)
-                return false;
-            __nanosleep(16);
-        }
-        return true;
-    };
+    // wait (bounded) until the chunk in stage st has been handed over
+    auto handed = [&](int st, uint32_t par) { return bounded_wait(&s_hand[st], par, limit); };
     // a solved row leaves: ring or scratch, neighbour's import ring; returns
     // where its global copy goes (written after the level's barrier)
     auto put = [&](bool upass, bool rm, int pos, int dst, int e, T acc) -> T * {
@@ -694,7 +723,7 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
         if (c == nL - 1) {
             // every y of the L pass is written before the gatherers read
             // the U pass's right-hand sides from them
-            consumer_sync_and(1);
+            solvers_sync_and<NT>(1);
             if (t == kThreads - 1)
                 mbar_arrive(ldone);
         }
@@ -702,170 +731,194 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
             st_release_cta_u32(&s_done, (uint32_t)(c + 1));
     };
     if constexpr (FW > 0) {
-        const int w = t / kWarpRows, lane = t % kWarpRows;
-        RowRegs<T, FW> A, B;
-        // one pass: chunks [c0, c1), U: the upper-triangular pass.  Before a
-        // level's barrier every thread has copied its row of the next chunk
-        // of the pass into registers, so that chunk's stage is free after
-        // the barrier, and the next level starts with its dependencies.
-        auto run = [&](auto Ucst, int c0, int c1) -> bool {
-            constexpr bool U = decltype(Ucst)::value;
-            if (c0 >= c1)
-                return false;
-            const bool rm = U ? blk.ring_U : blk.ring_L;
+        const int set = t / kThreads, lane = t % kWarpRows;
+        const int w = (t / kWarpRows) % kMaxWarps;
+        const int row = w * kWarpRows + lane;
+        volatile int *vfail = &s_err;
+#ifdef HEC_DEBUG
+        __shared__ int s_base; // position the program has reached in its pass
+        volatile int *vbase = &s_base;
+#endif
+        // One pass: chunks [c0, c1), U: the upper-triangular pass, RM: the
+        // dependencies are in the ring (else in the global scratch).  Set
+        // (c - c0) mod 2 solves chunk c.
+        auto run = [&](auto Ucst, auto RMcst, int c0, int c1) {
+            constexpr bool U = decltype(Ucst)::value, RM = decltype(RMcst)::value;
             const T *gdep = U ? zsc : ysc;
             T *scr = U ? zsc : ysc_w;
             const uint32_t imp = U ? imp_prev : imp_next;
-            // stage and handover count of the chunk after a given one
-            auto next = [&](int &st, uint32_t &h) {
-                if (++st == S) {
-                    st = 0;
-                    h += 32;
+            const uint32_t ring_a = smem_u32(ring);
+            RowRegs<T, FW> R;
+            uint32_t ya[FW]; // RM: shared addresses of the row's dependencies
+            uint32_t own_a = 0, exp_to = 0;
+            T *own = nullptr, *gout = nullptr;
+            T acc = T(0);
+            bool rows = false, mine = false, exports = false;
+            // copies this set's next chunk, c, in stage s, once it has been
+            // handed over, and forms every address its level will need
+            auto fetch = [&](int c) {
+                rows = mine = exports = false;
+                gout = nullptr;
+                if (*vfail)
+                    return;
+                if (!handed(s, hpar)) {
+                    *vfail = 1;
+                    return;
                 }
-            };
-            // the last thread confirms the handovers (acquire) before a
-            // barrier, so the other threads' loads after it need no check:
-            // chunks c0 and c0 + 1 now, chunk c + 2 at level c
-            int s1 = s, s2;
-            uint32_t h1 = hneed, h2;
-            next(s1, h1);
-            s2 = s1;
-            h2 = h1;
-            next(s2, h2);
-            int err = 0;
-            if (t == kThreads - 1)
-                err = !handed(s, hneed) || (c0 + 1 < c1 && !handed(s1, h1));
-            if (!consumer_sync_and(!err)) {
-                *verr = 1;
-                return true;
-            }
-            load_fixed<T, FW>(stages + (size_t)s * a.stage_bytes, rhs + (size_t)s * kThreads, w,
-                              lane, t, U, exps, A);
+                load_fixed<T, FW>(stages + (size_t)s * a.stage_bytes, rhs + (size_t)s * kThreads,
+                                  w, lane, U, exps, R);
+                rows = w < R.nwarps; // warps past the chunk's last one hold no rows
+                if (!rows)
+                    return;
 #ifdef HEC_DEBUG
-            int xbase = 0; // position the program has reached in its pass
-#endif
-            // level c: cur holds chunk c, nxt receives chunk c + 1; s, s1, s2
-            // are the stages of chunks c, c + 1, c + 2
-            auto level = [&](int c, RowRegs<T, FW> &cur, RowRegs<T, FW> &nxt) -> bool {
-                const bool more = c + 1 < c1, more2 = c + 2 < c1;
-                bool rows = w < cur.nwarps; // warps past the chunk's last one hold no rows
-#ifdef HEC_DEBUG
-                rows = rows && HEC_CHECK(cur.base == xbase, 4, c, cur.base, xbase) &&
-                       HEC_CHECK((cur.flags & 1) == (U ? 1 : 0), 1, c, cur.flags, nL) &&
-                       HEC_CHECK(cur.nrows >= 1 && cur.nrows <= kThreads &&
-                                     cur.nwarps == (cur.nrows + 31) / 32,
-                                 2, c, cur.nrows, cur.nwarps);
+                rows = rows && HEC_CHECK((R.flags & 1) == (U ? 1 : 0), 1, c, R.flags, nL) &&
+                       HEC_CHECK(R.nrows >= 1 && R.nrows <= kThreads &&
+                                     R.nwarps == (R.nrows + 31) / 32,
+                                 2, c, R.nrows, R.nwarps);
                 if (rows)
                     for (int k = 0; k < FW; ++k)
-                        rows &= rm ? HEC_CHECK(cur.d(k) >= 0 && cur.d(k) < nring, 5, c, cur.d(k),
-                                               nring)
-                                   : HEC_CHECK(cur.l(k) == T(0) ||
-                                                   (cur.d(k) >= 0 && cur.d(k) < cur.base),
-                                               6, c, cur.d(k), cur.base);
-                if (rows && t < cur.nrows && U)
-                    rows &= HEC_CHECK(cur.dst < a.n, 7, c, cur.dst, a.n);
-                xbase += cur.nrows;
+                        rows &= RM ? HEC_CHECK(R.d(k) >= 0 && R.d(k) < nring, 5, c, R.d(k), nring)
+                                   : HEC_CHECK(R.l(k) == T(0) ||
+                                                   (R.d(k) >= 0 && R.d(k) < R.base),
+                                               6, c, R.d(k), R.base);
+                if (rows && row < R.nrows && U)
+                    rows &= HEC_CHECK(R.dst < a.n, 7, c, R.dst, a.n);
+#else
+                (void)c;
 #endif
-                // this level's dependencies (the previous level's barrier has
-                // passed); padding lanes of the last warp carry valid slots
-                T y[FW];
-                if (rows) {
-                    if (rm) {
+                // padding lanes of the last warp carry valid slots
 #pragma unroll
-                        for (int k = 0; k < FW; ++k)
-                            y[k] = ring[cur.d(k)];
-                    } else {
-                        // global scratch: padding of a dependency-free row
-                        // points at a position this apply has not written (it
-                        // may hold NaN); entries of value 0 are not read
-#pragma unroll
-                        for (int k = 0; k < FW; ++k)
-                            y[k] = cur.l(k) != T(0) ? gdep[cur.d(k)] : T(0);
-                    }
-                }
-                // the next chunk's rows (handed over, confirmed before the
-                // previous barrier): loads only, first used after this barrier
-                if (more)
-                    load_fixed<T, FW>(stages + (size_t)s1 * a.stage_bytes,
-                                      rhs + (size_t)s1 * kThreads, w, lane, t, U, exps, nxt);
-                T out = T(0);
-                T *gout = nullptr;
-                if (rows) { // warps without rows issue no multiply-adds
-                    T acc = cur.rhs;
-#pragma unroll
-                    for (int k = 0; k < FW; ++k)
-                        acc = fma(-cur.l(k), y[k], acc);
-                    if (U)
-                        acc *= cur.dinv;
-                    if (t < cur.nrows) {
-                        const int pos = cur.base + t;
-                        if (rm)
-                            ring[pos & a.ring_mask] = acc;
-                        else
-                            scr[pos] = acc; // read by later levels of this pass
-                        if (U)
-                            gout = cur.dst >= 0 ? z + cur.dst : nullptr;
-                        else if (rm)
-                            gout = ysc_w + pos;
-                        if (cur.exp >= 0) // exports (-1 without export slots)
-                            st_cluster(imp + (uint32_t)((cur.exp & (RI - 1)) * sizeof(T)), acc);
-                        out = acc;
-                    }
-                }
-                int bad = 0;
-                if (t == kThreads - 1 && more2)
-                    bad = !handed(s2, h2);
-                if (!consumer_sync_and(!bad))
-                    return true; // a feeding warp's wait ran out
-                // every thread holds its rows of chunks c and c + 1: their
-                // stages are free (chunk c's only now at the pass's first level)
-                if (t == kThreads - 1) {
-                    if (c == c0)
-                        mbar_arrive(&empty[s]);
-                    if (more)
-                        mbar_arrive(&empty[s1]);
-                    if (signal)
-                        st_release_cta_u32(&s_done, (uint32_t)(c + 1));
-                }
-                if (gout)
-                    *gout = out;
-                s = s1;
-                hneed = h1;
-                s1 = s2;
-                h1 = h2;
-                next(s2, h2);
-                return false;
+                for (int k = 0; k < FW; ++k)
+                    ya[k] = ring_a + (uint32_t)(R.d(k) * sizeof(T));
+                mine = rows && row < R.nrows;
+                const int pos = R.base + row;
+                own_a = ring_a + (uint32_t)((pos & a.ring_mask) * sizeof(T));
+                own = scr + pos; // !RM: read by later levels
+                if (mine && U)
+                    gout = R.dst >= 0 ? z + R.dst : nullptr;
+                else if (mine && RM)
+                    gout = ysc_w + pos;
+                exports = mine && R.exp >= 0; // -1 without export slots
+                exp_to = imp + (uint32_t)((R.exp & (RI - 1)) * sizeof(T));
+                acc = R.rhs;
             };
-            for (int c = c0; c < c1; c += 2) {
-                if (level(c, A, B)) {
-                    *verr = 1;
-                    return true;
+            // solves chunk c: the previous level's barrier has passed
+            auto solve = [&]() {
+                if (!rows)
+                    return;
+                T y[FW];
+#pragma unroll
+                for (int k = 0; k < FW; ++k) {
+                    // global scratch: padding of a dependency-free row
+                    // points at a position this apply has not written (it
+                    // may hold NaN); entries of value 0 are not read
+                    if constexpr (RM)
+                        lds(ya[k], y[k]);
+                    else
+                        y[k] = R.l(k) != T(0) ? gdep[R.d(k)] : T(0);
                 }
-                if (c + 1 < c1 && level(c + 1, B, A)) {
-                    *verr = 1;
-                    return true;
+#pragma unroll
+                for (int k = 0; k < FW; ++k)
+                    acc = fma(-R.l(k), y[k], acc);
+                if (U)
+                    acc *= R.dinv;
+                if (mine) {
+                    if constexpr (RM)
+                        sts(own_a, acc);
+                    else
+                        *own = acc;
                 }
+                if (exports)
+                    st_cluster(exp_to, acc);
+            };
+            // the next chunk's stage and handover parity
+            auto advance = [&]() {
+                if (++s == S) {
+                    s = 0;
+                    hpar ^= 1u;
+                }
+            };
+            // the stage of a chunk copied before the last barrier is free
+            auto free_stage = [&](int c) {
+                if (row == 0 && c < c1)
+                    mbar_arrive(&empty[s]);
+            };
+#ifdef HEC_DEBUG
+            if (t == 0)
+                s_base = 0;
+#endif
+            int c = c0 + set; // the chunk this set solves next, in stage s
+            if (set == 0)
+                fetch(c);
+            solvers_sync<NT>();
+            if (set == 0) {
+                free_stage(c);
+                advance();
+            } else { // level c0 belongs to set 0
+                advance();
+                if (c < c1)
+                    fetch(c);
+                solvers_sync<NT>();
+                free_stage(c);
+                advance();
             }
-            return false;
+            while (c < c1) {
+                // ---- level c: this set solves
+#ifdef HEC_DEBUG
+                if (rows && lane == 0)
+                    HEC_CHECK(R.base == *vbase, 4, c, R.base, *vbase);
+                solvers_set_sync(set);
+                if (rows && row == 0)
+                    *vbase = R.base + R.nrows;
+#endif
+                solve();
+                solvers_sync<NT>();
+                // ---- level c + 1: the other set solves, this one fetches
+                if (signal && row == 0)
+                    st_release_cta_u32(&s_done, (uint32_t)(c + 1));
+                if (gout)
+                    *gout = acc;
+                if (c + 1 >= c1)
+                    break;
+                advance();
+                if (c + 2 < c1)
+                    fetch(c + 2);
+                solvers_sync<NT>();
+                free_stage(c + 2);
+                advance();
+                c += 2;
+            }
         };
-
-        if (run(std::integral_constant<bool, false>(), 0, nL)) {
-            failed = 1;
-        } else {
-            if (nL > 0) {
-                // every y of the L pass is written before the gatherers read
-                // the U pass's right-hand sides from them
-                consumer_sync_and(1);
-                if (t == kThreads - 1)
-                    mbar_arrive(ldone);
+        auto pass = [&](auto Ucst, int c0, int c1) {
+            constexpr bool U = decltype(Ucst)::value;
+            const int s0 = s;
+            const uint32_t h0 = hpar;
+            if (c0 < c1) {
+                if (U ? blk.ring_U : blk.ring_L)
+                    run(Ucst, std::true_type(), c0, c1);
+                else
+                    run(Ucst, std::false_type(), c0, c1);
             }
-            if (run(std::integral_constant<bool, true>(), nL, nch))
-                failed = 1;
+            // both sets go on from the stage after the pass's last chunk
+            const int n = s0 + (c1 - c0);
+            s = n % S;
+            hpar = h0 ^ ((uint32_t)(n / S) & 1u);
+        };
+        pass(std::false_type(), 0, nL);
+        if (nL > 0) {
+            // every y of the L pass is written before the gatherers read
+            // the U pass's right-hand sides from them
+            solvers_sync<NT>();
+            if (t == 0)
+                mbar_arrive(ldone);
         }
+        pass(std::true_type(), nL, nch);
+        solvers_sync<NT>();
+        failed = *vfail;
 
     } else {
         for (int c = 0; c < nch; ++c) {
-            if (!handed(s, hneed)) {
+            if (!handed(s, hpar)) {
                 err = 1;
                 *verr = 1;
             }
@@ -883,7 +936,7 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
                     out = acc;
                 }
             }
-            if (!consumer_sync_and(!err)) {
+            if (!solvers_sync_and<NT>(!err)) {
                 failed = 1; // the feeding warps' own waits run out
                 break;
             }
@@ -892,14 +945,14 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
             close(c, gout, out);
             if (++s == S) {
                 s = 0;
-                hneed += 32;
+                hpar ^= 1u;
             }
         }
     }
     }
     // every role has left its loop: drain the copies still in flight, report
     __syncthreads();
-    if (t == kThreads) {
+    if (t == NT) {
         const int issued = s_issued;
         const int first = issued - S > 0 ? issued - S : 0;
         for (int c = first; c < issued; ++c)
@@ -924,12 +977,16 @@ __global__ void __launch_bounds__(kThreads + kFeedThreads, 1) k_trsv_ras(TrsvArg
 // own slot and its dependencies are the slots of its columns (local row
 // indices), so there are no gatherer warps, no global scratch and no handover
 // counters: one issuer warp streams the chunks (rows of one level) into the
-// stages S chunks ahead with cp.async.bulk, and the solving warps run
-//   level c: read the dependencies and the right-hand side of chunk c's rows
-//            from xs, copy chunk c + 1's rows into registers, run the
-//            multiply-add chain, store the results into xs; the last thread
-//            confirms that chunk c + 2 has landed; barrier; chunk c + 1's stage
-//            is released.
+// stages S chunks ahead with cp.async.bulk, and three sets of solving warps
+// take the chunks in turn:
+//   level c: one set reads the dependencies and the right-hand side of chunk
+//            c's rows from xs, runs the multiply-add chain and stores the
+//            results into xs; the set whose chunk is c + 1 unpacks its slots
+//            into shared addresses; the set whose chunk is c + 2 confirms that
+//            its group has landed and copies its rows into registers; barrier
+//            of all sets.
+// (One set that did all of it spent 278 cycles a level solving and 680 on the
+// next chunk.  64^2, ILU(0), one block, FP64 apply: 88.7 -> 47.1 us.)
 // The per-level critical path is a shared-memory load, the row's dependent
 // multiply-adds (for U, the multiply by 1/u_ii) and a barrier of the solving
 // warps.  This is the latency-first form for small systems (a single ILU block
@@ -951,75 +1008,14 @@ template <class T, int FW> struct Res {
     __device__ static constexpr int block() { return dinv() + 32 * (int)sizeof(T); }
 };
 
-template <class T, int FW> struct ResRow {
-    int nrows, nwarps, flags;
-    int next_off, next_nw; // the next chunk's offset in its group's stage and its warps
-    typename Vec16<T>::type lv[Res<T, FW>::NV];
-    uint4 iv[Res<T, FW>::NI];
-    T dinv;
-    __device__ T l(int k) const { return Vec16<T>::get(lv[k / Res<T, FW>::VW], k % Res<T, FW>::VW); }
-    // uint16 k of the index vectors: dependency slot k < FW, the row's slot at FW
-    __device__ int slot(int k) const
-    {
-        const uint4 &v = iv[k / 8];
-        const int q = (k % 8) / 2;
-        const uint32_t word = q == 0 ? v.x : q == 1 ? v.y : q == 2 ? v.z : v.w;
-        return (int)((word >> (16 * (k % 2))) & 0xffffu);
-    }
-};
-
-// A solving thread's row of a resident-format chunk.  Every chunk has a block
-// for each of the kernel's NW solving warps (padding rows beyond its rows), so
-// a warp reads its block without waiting for the chunk's header; nw limits
-// the reads all the same (the header's warp count of a chunk is at most NW).
-template <class T, int FW, bool U>
-__device__ __forceinline__ void load_res(const unsigned char *ch, int w, int lane, int nw,
-                                         ResRow<T, FW> &R)
-{
-    using F = Res<T, FW>;
-    const int4 hdr = *reinterpret_cast<const int4 *>(ch);
-    const int4 nxt = *reinterpret_cast<const int4 *>(ch + 16);
-    R.nrows = hdr.x;
-    R.nwarps = hdr.y;
-    R.flags = hdr.w;
-    R.next_off = nxt.x;
-    R.next_nw = nxt.y;
-    if (w >= nw)
-        return;
-    const unsigned char *blk = ch + kFixedHeader + (size_t)w * F::block();
-    const typename Vec16<T>::type *val = reinterpret_cast<const typename Vec16<T>::type *>(blk) + lane;
-#pragma unroll
-    for (int v = 0; v < F::NV; ++v)
-        R.lv[v] = val[v * 32];
-    const uint4 *idx = reinterpret_cast<const uint4 *>(blk + F::idx()) + lane;
-#pragma unroll
-    for (int v = 0; v < F::NI; ++v)
-        R.iv[v] = idx[v * 32];
-    if (U)
-        R.dinv = reinterpret_cast<const T *>(blk + F::dinv())[lane];
-}
-
-// Barrier of the NT solving threads of a resident-kernel CTA (named barrier
-// 1), AND-reducing a flag.
-template <int NT> __device__ __forceinline__ int solvers_sync_and(int flag)
-{
-    int all;
-    asm volatile("{\n\t.reg .pred p, q;\n\t"
-                 "setp.ne.s32 p, %1, 0;\n\t"
-                 "barrier.cta.red.and.pred q, 1, %2, p;\n\t"
-                 "selp.s32 %0, 1, 0, q;\n\t}"
-                 : "=r"(all)
-                 : "r"(flag), "n"(NT)
-                 : "memory");
-    return all;
-}
-
-// NW solving warps (chunks of at most 32 NW rows, NW sized at setup to the
-// widest level) and one issuer warp.
+// Three sets of NW solving warps (chunks of at most 32 NW rows, NW sized at
+// setup to the widest level) and one issuer warp.
+constexpr int kResSets = 3;
+template <int NW> constexpr int kResSolvers = kResSets * NW * 32;
 template <class T, int FW, int NW>
-__global__ void __launch_bounds__(NW * 32 + 32, 1) k_trsv_res(TrsvArgs a)
+__global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a)
 {
-    constexpr int NT = NW * 32; // solving threads
+    constexpr int NT = kResSolvers<NW>; // solving threads
     extern __shared__ __align__(128) unsigned char smem[];
     count_launch(a.st);
     if (a.st && a.st->skip)
@@ -1041,13 +1037,14 @@ __global__ void __launch_bounds__(NW * 32 + 32, 1) k_trsv_res(TrsvArgs a)
     const bool stall_test = a.spin_limit < 0; // fault injection: nothing is issued
     const long long limit = stall_test ? -a.spin_limit : a.spin_limit;
     const int t = threadIdx.x;
-    __shared__ int s_issued;
+    __shared__ int s_issued, s_fail;
     if (t == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
         s_issued = 0;
+        s_fail = 0;
         fence_mbar_init();
     }
     __syncthreads();
@@ -1061,114 +1058,161 @@ __global__ void __launch_bounds__(NW * 32 + 32, 1) k_trsv_res(TrsvArgs a)
     } else {
         // ------------------------------------------------------------ solving warps
         // r on V_b into the resident vector; slot nv holds 0 (padding)
-        for (int i = t; i < blk.nv; i += NT) {
-            const int g = vrows[i];
-            xs[i] = HEC_CHECK(g >= 0 && g < a.n, 3, 0, g, a.n) ? r[g] : T(0);
+        // (kBatch rows' loads in flight)
+        constexpr int kBatch = 8;
+        for (int i0 = t; i0 < blk.nv; i0 += kBatch * NT) {
+            int g[kBatch];
+            T v[kBatch];
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q)
+                g[q] = i0 + q * NT < blk.nv ? vrows[i0 + q * NT] : -1;
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q)
+                v[q] = i0 + q * NT < blk.nv && HEC_CHECK(g[q] >= 0 && g[q] < a.n, 3, 0, g[q], a.n)
+                           ? r[g[q]]
+                           : T(0);
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q)
+                if (i0 + q * NT < blk.nv)
+                    xs[i0 + q * NT] = v[q];
         }
         if (t == 0)
             xs[blk.nv] = T(0);
-        const int w = t / kWarpRows, lane = t % kWarpRows;
+        // each set's warps are turned by one more, so that the sets' chunks of
+        // few warps use other sub-partitions of the SM
+        const int set = t / (NW * 32), lane = t % kWarpRows;
+        const int w = (t / kWarpRows + set) % NW;
+        const int row = w * kWarpRows + lane;
         // Chunks arrive in groups of G (one bulk copy each) in stage order, all
         // of one size CB: chunk k of a group sits at k CB in its group's stage.
-        // A chunk's place is that stage s, the stage's phase parity and k.
+        // A chunk's place is that stage ls, the stage's phase parity lph and lk.
         constexpr int CB = kFixedHeader + NW * Res<T, FW>::block();
         const int G = a.res_group;
-        struct Loc {
-            int s;
-            uint32_t ph;
-            int k;
-        };
-        auto next = [&](Loc l) -> Loc {
-            if (++l.k == G) {
-                l.k = 0;
-                if (++l.s == S) {
-                    l.s = 0;
-                    l.ph ^= 1u;
+        const uint32_t xs_a = smem_u32(xs);
+        volatile int *vfail = &s_fail;
+        int ls = 0, lk = 0; // the place of this set's next chunk
+        uint32_t lph = 0;
+        auto advance = [&](int n) {
+            for (lk += n; lk >= G; lk -= G)
+                if (++ls == S) {
+                    ls = 0;
+                    lph ^= 1u;
                 }
+        };
+        using F = Res<T, FW>;
+        typename Vec16<T>::type lv[F::NV];
+        uint4 iv[F::NI];
+        T dinv = T(0);
+        int nrows = 0;
+        uint32_t xa[FW + 1]; // shared addresses of the dependencies and the own slot
+        bool rows = false, mine = false, upper = false;
+        // copies this set's next chunk, at (ls, lph, lk), once its group has
+        // landed (after the first barrier, only the chunk that opens a group
+        // asks: the other sets copy from it in later levels)
+        auto fetch = [&](bool ask) {
+            rows = false;
+            if (*vfail) // a group that never landed: nothing is read from it
+                return;
+            if (ask && !bounded_wait(&full[ls], lph, limit)) {
+                *vfail = 1;
+                return;
             }
-            return l;
-        };
-        auto landed = [&](const Loc &l) -> bool { return bounded_wait(&full[l.s], l.ph, limit); };
-        auto load = [&](bool U, const Loc &l, ResRow<T, FW> &R) {
-            const unsigned char *ch = stages + (size_t)l.s * a.stage_bytes + (size_t)l.k * CB;
-            if (U)
-                load_res<T, FW, true>(ch, w, lane, NW, R);
-            else
-                load_res<T, FW, false>(ch, w, lane, NW, R);
-        };
-        const Loc l0{0, 0u, 0};
-        int bad = 0;
-        if (t == NT - 1 && nch > 0)
-            bad = !landed(l0);
-        // the gather above is complete and the first group has landed
-        if (!solvers_sync_and<NT>(!bad)) {
-            failed = 1;
-        } else if (nch > 0) {
-            ResRow<T, FW> A, B;
-            load(0 >= nL, l0, A);
-            Loc ln = next(l0); // chunk 1
-            bad = (t == NT - 1 && nch > 1 && ln.k == 0) ? !landed(ln) : 0;
-            if (!solvers_sync_and<NT>(!bad))
-                failed = 1;
-            // level c: cur holds chunk c's rows, nxt receives chunk c + 1's
-            // (found at ln); every place is known without reading a header
-            auto level = [&](int c, ResRow<T, FW> &cur, ResRow<T, FW> &nxt) -> bool {
-                const bool U = c >= nL;
-                const bool rows = w < cur.nwarps; // warps past the chunk's last one idle
-                T y[FW];
-                T acc = T(0);
-                int me = blk.nv;
-                if (rows) {
+            const unsigned char *ch = stages + (size_t)ls * a.stage_bytes + (size_t)lk * CB;
+            const int2 hdr = *reinterpret_cast<const int2 *>(ch); // rows, warps
+            const unsigned char *blkp = ch + kFixedHeader + (size_t)w * F::block();
 #pragma unroll
-                    for (int k = 0; k < FW; ++k) {
-                        const int d = cur.slot(k);
-                        y[k] = HEC_CHECK(d <= blk.nv, 5, c, d, blk.nv) ? xs[d] : T(0);
-                    }
-                    me = cur.slot(FW);
-                    if (!HEC_CHECK(me <= blk.nv, 7, c, me, blk.nv))
-                        me = blk.nv;
-                    acc = xs[me];
-                }
-                const Loc l2 = next(ln); // chunk c + 2
-                const bool more = c + 1 < nch;
-                if (more) // its group landed: confirmed before the previous barrier
-                    load(c + 1 >= nL, ln, nxt);
-                // chunk c + 2 opens a group: the last thread confirms it landed
-                int late = 0;
-                if (t == NT - 1 && c + 2 < nch && l2.k == 0)
-                    late = !landed(l2);
-                if (rows) {
+            for (int v = 0; v < F::NV; ++v)
+                lv[v] = (reinterpret_cast<const typename Vec16<T>::type *>(blkp) + lane)[v * 32];
 #pragma unroll
-                    for (int k = 0; k < FW; ++k)
-                        acc = fma(-cur.l(k), y[k], acc);
-                    if (U)
-                        acc *= cur.dinv;
-                    if (t < cur.nrows && me < blk.nv)
-                        xs[me] = acc;
-                }
-                if (!solvers_sync_and<NT>(!late))
-                    return false;
-                // every thread holds chunks up to c + 1 in registers: the group
-                // that chunk closes has a free stage
-                if (t == NT - 1) {
-                    if (c == 0 && (G == 1 || nch == 1))
-                        mbar_arrive(&empty[0]);
-                    if (more && (ln.k == G - 1 || c + 1 == nch - 1))
-                        mbar_arrive(&empty[ln.s]);
-                }
-                ln = l2;
-                return true;
-            };
-            for (int c = 0; c < nch && !failed; c += 2) {
-                if (!level(c, A, B))
-                    failed = 1;
-                else if (c + 1 < nch && !level(c + 1, B, A))
-                    failed = 1;
+            for (int v = 0; v < F::NI; ++v)
+                iv[v] = (reinterpret_cast<const uint4 *>(blkp + F::idx()) + lane)[v * 32];
+            dinv = reinterpret_cast<const T *>(blkp + F::dinv())[lane];
+            nrows = hdr.x;
+            rows = w < hdr.y; // warps past the chunk's last one idle
+        };
+        // chunk c's slots as shared addresses; the chunk that opens a group
+        // frees the stage of the one before (its last chunk was copied at least
+        // a barrier ago)
+        auto prepare = [&](int c) {
+            if (row == 0 && lk == 0 && c > 0 && c < nch)
+                mbar_arrive(&empty[ls == 0 ? S - 1 : ls - 1]);
+#pragma unroll
+            for (int k = 0; k <= FW; ++k) { // vectors of 8 uint16
+                const uint4 v = iv[k / 8];
+                const uint32_t word = (k % 8) / 2 == 0 ? v.x : (k % 8) / 2 == 1 ? v.y
+                                      : (k % 8) / 2 == 2 ? v.z : v.w;
+                uint32_t sl = (word >> (16 * (k % 2))) & 0xffffu;
+#ifdef HEC_DEBUG
+                if (rows && !HEC_CHECK(sl <= (uint32_t)blk.nv, k < FW ? 5 : 7, c, sl, blk.nv))
+                    sl = blk.nv;
+#endif
+                xa[k] = xs_a + sl * (uint32_t)sizeof(T);
             }
-            if (!failed)
-                for (int i = blk.own0 + t; i < blk.own1; i += NT)
-                    z[vrows[i]] = xs[i];
+            mine = rows && row < nrows && xa[FW] < xs_a + blk.nv * (uint32_t)sizeof(T);
+            upper = c >= nL;
+        };
+        int c = set; // the chunk this set solves next
+        advance(set);
+        // before level 0: its chunk is ready, the next one copied
+        if (set < 2 && c < nch)
+            fetch(true);
+        if (set == 0)
+            prepare(c);
+        // the gather above is complete too
+        solvers_sync<NT>();
+        for (int l = 0; l < c && l < nch; ++l) { // the levels before this set's first
+            if (l == c - 1)
+                prepare(c);
+            else if (c < nch)
+                fetch(lk == 0);
+            solvers_sync<NT>();
         }
+        while (c < nch) {
+            // ---- level c
+            if (rows) {
+                T y[FW], acc;
+#pragma unroll
+                for (int k = 0; k < FW; ++k)
+                    lds(xa[k], y[k]);
+                lds(xa[FW], acc);
+#pragma unroll
+                for (int k = 0; k < FW; ++k)
+                    acc = fma(-Vec16<T>::get(lv[k / F::VW], k % F::VW), y[k], acc);
+                if (upper)
+                    acc *= dinv;
+                if (mine)
+                    sts(xa[FW], acc);
+            }
+            solvers_sync<NT>();
+            // ---- level c + 1
+            if (c + 1 >= nch)
+                break;
+            advance(kResSets);
+            if (c + kResSets < nch)
+                fetch(lk == 0);
+            else
+                rows = false;
+            solvers_sync<NT>();
+            // ---- level c + 2
+            if (c + 2 >= nch)
+                break;
+            prepare(c + kResSets);
+            solvers_sync<NT>();
+            c += kResSets;
+        }
+        solvers_sync<NT>();
+        failed = *vfail;
+        if (!failed)
+            for (int i0 = blk.own0 + t; i0 < blk.own1; i0 += kBatch * NT) {
+                int g[kBatch];
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q)
+                    g[q] = i0 + q * NT < blk.own1 ? vrows[i0 + q * NT] : -1;
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q)
+                    if (i0 + q * NT < blk.own1)
+                        z[g[q]] = xs[i0 + q * NT];
+            }
     }
     // every role has left its loop: drain the copies still in flight, report
     __syncthreads();
@@ -1225,7 +1269,7 @@ template <class T, int FW> static int launch_t(const TrsvArgs &a, cudaStream_t s
         return -1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)a.nblocks);
-    cfg.blockDim = dim3(kThreads + kFeedThreads);
+    cfg.blockDim = dim3(kSolvers<FW> + kFeedThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -1243,7 +1287,7 @@ template <class T, int FW, int NW> static int launch_res(const TrsvArgs &a, cuda
     const size_t smem = trsv_res_smem_bytes(a.stage_bytes, a.nstages, a.res_slots, sizeof(T));
     if (prepare_trsv<T, FW, true, NW>() != cudaSuccess)
         return -1;
-    k_trsv_res<T, FW, NW><<<a.nblocks, NW * 32 + 32, smem, s>>>(a);
+    k_trsv_res<T, FW, NW><<<a.nblocks, kResSolvers<NW> + 32, smem, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

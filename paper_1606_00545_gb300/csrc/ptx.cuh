@@ -128,6 +128,25 @@ __device__ __forceinline__ void fence_proxy_async_global()
     asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
+// Loads and stores of shared memory by 32-bit shared address (formed ahead of
+// a barrier, so that nothing but the access follows it).
+__device__ __forceinline__ void lds(uint32_t a, double &v)
+{
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void lds(uint32_t a, float &v)
+{
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void sts(uint32_t a, double v)
+{
+    asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void sts(uint32_t a, float v)
+{
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
 // ------------------------------------------------------------------ clusters
 // Barrier of every thread of the cluster (all threads must reach it); the
 // release/acquire pair orders each CTA's earlier shared-memory writes before

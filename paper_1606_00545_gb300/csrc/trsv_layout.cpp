@@ -1074,10 +1074,19 @@ int pack_trsv(const std::vector<BlockFactor> &Bs, int n, int stage_bytes, int ma
         emit_block(Bs[b], plans[b], R, std::max(RI, 1), vb, uniform_width, exps, nparts, outs[b]);
     });
 
+    // a stage holds the largest chunk planned, so that as many stages as
+    // possible fit (the kernel keeps copies and gathers of several chunks in
+    // flight)
+    size_t most_bytes = 16;
+    for (const BlockOut &O : outs)
+        for (const std::vector<uint2> &cs : O.chunks)
+            for (const uint2 &c : cs)
+                most_bytes = std::max(most_bytes, (size_t)c.y);
+
     P.pack.clear();
     P.chunks.clear();
     P.parts = nparts;
-    P.stage_bytes = stage_bytes;
+    P.stage_bytes = (int)((most_bytes + 127) & ~(size_t)127);
     P.exp_arrays = exps && uniform_width > 0 ? 1 : 0;
     P.ring_slots = R;
     P.import_slots = RI;
