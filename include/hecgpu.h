@@ -364,8 +364,11 @@ int hec_precond_set_trsv_parts(hec_precond_t M, int32_t parts);
  *     holds more than 128 rows and the streamed kernel would not split a
  *     block over several CTAs (measured on GB300: 1.1-1.2x faster there,
  *     slower on wider levels), else streamed.
- * The FP32 layout of the mixed-precision mode follows the same rule.  Call
- * it between ilu_k_setup and level_schedule; HEC_ERR_INVALID afterwards,
+ * The FP32 layout of the mixed-precision mode follows the same rule; under
+ * HEC_TRSV_AUTO, FP32 factors with rows of more than 8 entries whose blocks
+ * fit in shared memory and would not be split run a third, long-row kernel
+ * (hec_precond_get_layout still returns their streamed layout).  Call it
+ * between ilu_k_setup and level_schedule; HEC_ERR_INVALID afterwards,
  * for a damped-Jacobi handle or another value; level_schedule returns
  * HEC_ERR_INVALID when HEC_TRSV_RESIDENT is asked for and a block does not
  * fit. */

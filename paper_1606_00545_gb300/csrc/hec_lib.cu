@@ -390,12 +390,12 @@ int layout_parts(const hec_precond_s *M, int idx)
 // fixed-slot formats (0: generic) and, for the resident layout, the stage
 // count (the streamed kernel's is sized at upload).
 int pack_layout(const hec_precond_s *M, int idx, TrsvPack &P, int &fixed_width, int &nstages,
-                std::string &msg)
+                std::string &msg, bool streamed = false)
 {
     const int vb = idx == 0 ? 8 : 4;
     const int longest =
         std::max(max_factor_width(M->blocks, false), max_factor_width(M->blocks, true));
-    if (M->trsv_kernel != HEC_TRSV_STREAMED) {
+    if (M->trsv_kernel != HEC_TRSV_STREAMED && !streamed) {
         const int rw = trsv_resident_width(longest);
         int maxnv = 0, widest = 0;
         for (const BlockFactor &B : M->blocks) {
@@ -423,6 +423,20 @@ int pack_layout(const hec_precond_s *M, int idx, TrsvPack &P, int &fixed_width, 
             if (nstages > 0) {
                 fixed_width = rw;
                 return HEC_OK;
+            }
+        }
+        // Rows too long for the fixed-slot formats, FP32: the long-row kernel
+        // where the block's vector fits beside three stages and the streamed
+        // kernel would not split a block.  LRULE
+        if (M->trsv_kernel == HEC_TRSV_AUTO && idx == 1 && trsv_uniform_width(longest) == 0 &&
+            maxnv < kLongSlots && layout_parts(M, idx) == 1) {
+            const int stage = kLongWarps * kLongUnit;
+            nstages = M->host_only
+                          ? (trsv_res_smem_bytes(stage, 3, maxnv + 1, vb) <= 226 * 1024 ? 3 : 0)
+                          : trsv_res_stages_for(stage, maxnv + 1, vb);
+            if (nstages > 0) {
+                fixed_width = 0;
+                return pack_trsv_long(M->blocks, P, msg);
             }
         }
         if (M->trsv_kernel == HEC_TRSV_RESIDENT) {
@@ -1365,6 +1379,7 @@ int refactor_precond(hec_matrix_s *A, hec_precond_s *M, cudaStream_t s)
         fa.rm_len = L.d_rml.as<int>();
         fa.rm_diag = L.d_rmd.as<int>();
         fa.f = M->rf_f.as<double>();
+        fa.long_rows = L.pack.resident == 2;
         launch_fill_pack(fa, (int)L.pack.chunks.size(), idx == 1, s);
         HEC_TRY(check_launch("fill"));
     }
@@ -1874,7 +1889,16 @@ int hec_precond_get_layout(hec_precond_t M, int32_t fp32, int64_t *pack_bytes, i
             return fail(HEC_ERR_INVALID, "level_schedule has not run");
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         HEC_TRY(build_layout(M, fp32, s));
-        const TrsvLayout &L = M->lay[fp32];
+        TrsvLayout streamed; // the long-row kernel's units are not this format: packed for the query
+        if (M->lay[fp32].pack.resident == 2) {
+            HEC_TRY(refresh_host_factors(M, s));
+            std::string msg;
+            int ns = 0;
+            const int rc = pack_layout(M, fp32, streamed.pack, streamed.fixed_width, ns, msg, true);
+            if (rc != HEC_OK)
+                return fail(rc, "%s", msg.c_str());
+        }
+        const TrsvLayout &L = M->lay[fp32].pack.resident == 2 ? streamed : M->lay[fp32];
         int64_t total = 0;
         for (const uint2 &c : L.pack.chunks)
             total = std::max<int64_t>(total, (int64_t)c.x * 16 + c.y);

@@ -79,7 +79,7 @@ struct TrsvPack {
     std::vector<int> rm_start, rm_len, rm_diag; // first value's entry, count, diagonal (U; -1 for L)
     // resident-vector layout (pack_trsv_resident): one CTA per block, the
     // block's vector in shared memory
-    int resident = 0;
+    int resident = 0;           // 1: pack_trsv_resident, 2: pack_trsv_long
     int res_slots = 0;          // largest block's rows + 1
     int res_warps = 0;          // solving warps of the kernel (2, 4 or 8): chunks of 32 x that rows
     int res_group = 1;          // chunks per group (one bulk copy; every chunk the same size)
@@ -100,6 +100,10 @@ int pack_trsv(const std::vector<BlockFactor> &B, int n, int stage_bytes, int max
 // row), dependencies as local row slots, every block below 65535 rows.
 int pack_trsv_resident(const std::vector<BlockFactor> &B, int width, int vb, TrsvPack &out,
                        std::string &msg);
+// The layout of k_trsv_long (FP32 values): blocks whose vector fits in shared
+// memory and whose rows are too long for the resident kernel; a row's entries
+// are spread over a group of lanes.  Every block below 65535 rows.
+int pack_trsv_long(const std::vector<BlockFactor> &B, TrsvPack &out, std::string &msg);
 // The resident width for rows of at most longest_row entries, 0 if none.
 int trsv_resident_width(int longest_row);
 // The parts per block worth launching: split while the widest block's levels

@@ -214,6 +214,25 @@ template <class T> __global__ void __launch_bounds__(kThreads) k_fill_pack(FillA
     }
 }
 
+// The same for the long-row kernel's units (kernels.cuh): a warp per unit.
+__global__ void __launch_bounds__(kThreads) k_fill_long(FillArgs a, int nunits)
+{
+    const int u = blockIdx.x * (kThreads / 32) + threadIdx.x / 32, lane = threadIdx.x % 32;
+    if (u >= nunits)
+        return;
+    unsigned char *ch = a.pack + (size_t)a.chunks[u].x * 16;
+    const int64_t q = a.chunk_row0[u] + lane;
+    const int start = a.rm_start[q], cnt = a.rm_len[q] & 0xff, G = a.rm_len[q] >> 8;
+    const int dg = a.rm_diag[q];
+    float v[kLongPerLane];
+#pragma unroll
+    for (int k = 0; k < kLongPerLane; ++k)
+        v[k] = k < cnt ? (float)a.f[start + k * G] : 0.0f;
+    reinterpret_cast<float4 *>(ch)[lane] = make_float4(v[0], v[1], v[2], v[3]);
+    if (dg >= 0)
+        reinterpret_cast<float *>(ch + 512 + 16 * lane)[3] = (float)__ddiv_rn(1.0, a.f[dg]);
+}
+
 __global__ void k_jacobi_dinv(int n, const double *val, const int64_t *diag, double omega,
                               double *dinv, float *dinv32, int *err)
 {
@@ -255,6 +274,11 @@ int launch_fill_pack(const FillArgs &a, int nchunks, bool fp32, cudaStream_t s)
 {
     if (nchunks <= 0)
         return 0;
+    if (a.long_rows) {
+        const int per = kThreads / 32;
+        k_fill_long<<<(nchunks + per - 1) / per, kThreads, 0, s>>>(a, nchunks);
+        return 0;
+    }
     if (fp32)
         k_fill_pack<float><<<nchunks, kThreads, 0, s>>>(a);
     else

@@ -1229,6 +1229,186 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
     }
 }
 
+// ------------------------------------------------------------------ long-row kernel
+// Blocks whose rows are too long for the resident kernel but whose FP32 vector
+// fits in shared memory: the vector is solved in place as there, and a row's
+// entries are spread over a group of lanes (4 a lane), summed by shuffles.  One
+// thread per row leaves a level of such a block with a handful of active lanes
+// and one long chain: the 27-point matrix with irregular rows has 17 rows in
+// the median level, 13 entries a row (up to 117), and its dependencies reach
+// further back than any ring, so the streamed kernel also read them from
+// global memory: 72^3, ILU(0), 64 blocks 1,806 -> 295 us.
+// A warp's work in a level is a unit (kernels.cuh); kLongWarps units, one per
+// warp, travel in one bulk copy.  A warp holds its next unit in registers with
+// its addresses formed, passes the level barriers that come before it, solves
+// it, passes its own level's barrier and then loads the next one -- a level of
+// three units leaves each warp several levels for that.
+constexpr int kLongThreads = 32 * kLongWarps;
+__global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
+{
+    constexpr int NT = kLongThreads;
+    extern __shared__ __align__(128) unsigned char smem[];
+    count_launch(a.st);
+    if (a.st && a.st->skip)
+        return; // uniform over the grid
+    const float *r = reinterpret_cast<const float *>(a.r);
+    if (a.r_from_j)
+        r += (int64_t)a.st->j * a.ldv;
+    float *z = reinterpret_cast<float *>(a.z);
+    const TrsvBlock blk = a.blocks[blockIdx.x];
+    const int S = a.nstages;
+    unsigned char *stages = smem;
+    float *xs = reinterpret_cast<float *>(smem + (size_t)S * a.stage_bytes);
+    uint64_t *full = reinterpret_cast<uint64_t *>(
+        reinterpret_cast<unsigned char *>(xs) + (((size_t)a.res_slots * sizeof(float) + 7) & ~(size_t)7));
+    uint64_t *empty = full + S;
+    const int ng = blk.ngroups, nlev = blk.ring_L;
+    const int *vrows = a.vrows + blk.yoff;
+    const bool stall_test = a.spin_limit < 0; // fault injection: nothing is issued
+    const long long limit = stall_test ? -a.spin_limit : a.spin_limit;
+    const int t = threadIdx.x;
+    __shared__ int s_issued, s_fail;
+    if (t == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], kLongWarps);
+        }
+        s_issued = 0;
+        s_fail = 0;
+        fence_mbar_init();
+    }
+    __syncthreads();
+    int failed = 0;
+    if (t >= NT) {
+        // ------------------------------------------------------------ issuer warp
+        if (!stall_test &&
+            !issue_chunks(a.groups + blk.zoff, ng, S, a.stage_bytes, a.pack, stages, full, empty,
+                          limit, t - NT, &s_issued))
+            failed = 1;
+    } else {
+        // ------------------------------------------------------------ solving warps
+        constexpr int kBatch = 8;
+        for (int i0 = t; i0 < blk.nv; i0 += kBatch * NT) {
+            int g[kBatch];
+            float v[kBatch];
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q)
+                g[q] = i0 + q * NT < blk.nv ? vrows[i0 + q * NT] : -1;
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q)
+                v[q] = i0 + q * NT < blk.nv && HEC_CHECK(g[q] >= 0 && g[q] < a.n, 3, 0, g[q], a.n)
+                           ? r[g[q]]
+                           : 0.0f;
+#pragma unroll
+            for (int q = 0; q < kBatch; ++q)
+                if (i0 + q * NT < blk.nv)
+                    xs[i0 + q * NT] = v[q];
+        }
+        if (t == 0)
+            xs[blk.nv] = 0.0f; // padding
+        const int w = t / 32, lane = t % 32;
+        const uint32_t xs_a = smem_u32(xs);
+        volatile int *vfail = &s_fail;
+        int s = 0; // the stage of the warp's next unit and its phase
+        uint32_t par = 0;
+        float4 val;
+        float mul = 1.0f;
+        uint32_t xa[kLongPerLane + 1]; // shared addresses of the dependencies and the own slot
+        int flags = 0;
+        // copies the unit of group g and forms its addresses; the stage is
+        // free once every warp has its unit
+        auto fetch = [&](int g) -> bool {
+            if (!bounded_wait(&full[s], par, limit)) {
+                *vfail = 1;
+                return false;
+            }
+            const unsigned char *u = stages + (size_t)s * a.stage_bytes + w * kLongUnit;
+            val = reinterpret_cast<const float4 *>(u)[lane];
+            const uint4 rec = reinterpret_cast<const uint4 *>(u + 512)[lane];
+            uint32_t sl[kLongPerLane + 1] = {rec.x & 0xffffu, rec.x >> 16, rec.y & 0xffffu,
+                                             rec.y >> 16, rec.z & 0xffffu};
+            flags = (int)(rec.z >> 16);
+            mul = __uint_as_float(rec.w);
+#pragma unroll
+            for (int k = 0; k <= kLongPerLane; ++k) {
+#ifdef HEC_DEBUG
+                if (!HEC_CHECK(sl[k] <= (uint32_t)blk.nv, k < kLongPerLane ? 5 : 7, g, sl[k], blk.nv))
+                    sl[k] = blk.nv;
+#endif
+                xa[k] = xs_a + sl[k] * 4u;
+            }
+            (void)g;
+            __syncwarp();
+            if (lane == 0)
+                mbar_arrive(&empty[s]);
+            if (++s == S) {
+                s = 0;
+                par ^= 1u;
+            }
+            return true;
+        };
+        int passed = 0;
+        bool have = ng > 0 && fetch(0);
+        solvers_sync<NT>(); // the gather above is complete
+        for (int g = 0; g < ng && have; ++g) {
+            for (int nb = (flags >> 7) & 63; nb > 0; --nb, ++passed)
+                solvers_sync<NT>();
+            float y[kLongPerLane], acc, x;
+#pragma unroll
+            for (int k = 0; k < kLongPerLane; ++k)
+                lds(xa[k], y[k]);
+            lds(xa[kLongPerLane], x);
+            acc = (flags & 64) ? x : 0.0f; // the row's first lane holds its right-hand side
+            acc = fmaf(-val.x, y[0], acc);
+            acc = fmaf(-val.y, y[1], acc);
+            acc = fmaf(-val.z, y[2], acc);
+            acc = fmaf(-val.w, y[3], acc);
+            const int lg = flags & 7, maxlg = (flags >> 3) & 7;
+            for (int q = 0; q < maxlg; ++q) {
+                const float o = __shfl_xor_sync(0xffffffffu, acc, 1 << q);
+                acc += q < lg ? o : 0.0f;
+            }
+            if (flags & 64)
+                sts(xa[kLongPerLane], acc * mul);
+            if (flags >> 13 & 1) { // the level goes on without this warp
+                solvers_sync<NT>();
+                ++passed;
+            }
+            if (g + 1 < ng)
+                have = fetch(g + 1);
+        }
+        // every warp passes every level's barrier, also after a failed wait
+        for (; passed < nlev; ++passed)
+            solvers_sync<NT>();
+        solvers_sync<NT>();
+        failed = *vfail;
+        if (!failed)
+            for (int i0 = blk.own0 + t; i0 < blk.own1; i0 += kBatch * NT) {
+                int g[kBatch];
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q)
+                    g[q] = i0 + q * NT < blk.own1 ? vrows[i0 + q * NT] : -1;
+#pragma unroll
+                for (int q = 0; q < kBatch; ++q)
+                    if (i0 + q * NT < blk.own1)
+                        z[g[q]] = xs[i0 + q * NT];
+            }
+    }
+    // every role has left its loop: drain the copies still in flight, report
+    __syncthreads();
+    if (t == NT) {
+        const int issued = s_issued;
+        const int first = issued - S > 0 ? issued - S : 0;
+        for (int c = first; c < issued; ++c)
+            bounded_wait(&full[c % S], (uint32_t)(c / S) & 1u, kDrainPolls);
+    }
+    if (failed) {
+        atomicExch(a.err, HEC_ERR_TIMEOUT);
+        if (a.st)
+            a.st->err = HEC_ERR_TIMEOUT;
+    }
+}
+
 // The dynamic shared memory limit is a process-wide attribute of the kernel:
 // raised once to the device's opt-in maximum, so that launches of different
 // sizes from several host threads never race on it.
@@ -1291,6 +1471,28 @@ template <class T, int FW, int NW> static int launch_res(const TrsvArgs &a, cuda
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+static int launch_long(const TrsvArgs &a, cudaStream_t s)
+{
+    static std::once_flag once;
+    static cudaError_t e = cudaSuccess;
+    std::call_once(once, []() {
+        int dev = 0, optin = 0;
+        cudaGetDevice(&dev);
+        cudaFuncAttributes fa{};
+        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess)
+            e = cudaFuncGetAttributes(&fa, k_trsv_long);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_trsv_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     optin - (int)fa.sharedSizeBytes);
+    });
+    if (e != cudaSuccess)
+        return -1;
+    const size_t smem = trsv_res_smem_bytes(a.stage_bytes, a.nstages, a.res_slots, sizeof(float));
+    k_trsv_long<<<a.nblocks, kLongThreads + 32, smem, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
 template <class T, int FW> static int launch_res_w(const TrsvArgs &a, cudaStream_t s)
 {
     switch (a.res_warps) {
@@ -1343,6 +1545,8 @@ bool trsv_debug_build()
 
 int launch_trsv(const TrsvArgs &a, cudaStream_t s, bool fp32)
 {
+    if (a.resident == 2)
+        return fp32 ? launch_long(a, s) : -1;
     if (a.resident) {
 #define HEC_RES_CASE(W)                                                                          \
     case W: return fp32 ? launch_res_w<float, W>(a, s) : launch_res_w<double, W>(a, s);

@@ -199,7 +199,8 @@ struct TrsvArgs {
     int n;                      // rows of z (bounds checks of the debug build)
     int r_from_j;
     int64_t ldv;
-    int resident;               // 1: the resident-vector kernel (fixed_width: its row width)
+    int resident;               // 1: the resident-vector kernel (fixed_width: its row width);
+                                // 2: the long-row kernel (FP32)
     int res_slots;              // resident kernel: shared-memory vector slots (largest nv + 1)
     const int *vrows;           // resident kernel: V_b of every block, concatenated
     const uint2 *groups;        // resident kernel: chunk groups {offset / 16, bytes}
@@ -217,6 +218,24 @@ size_t trsv_res_smem_bytes(int stage_bytes, int nstages, int res_slots, int vbyt
 // Largest stage count (3..8) that fits, 0 if even 3 stages do not.
 int trsv_res_stages_for(int stage_bytes, int res_slots, int vbytes);
 int launch_trsv(const TrsvArgs &a, cudaStream_t s, bool fp32 = false);
+// The long-row kernel's units (trsv_layout.cpp writes them, k_trsv.cu reads
+// them, k_refactor.cu refills their values).  A unit is one warp's work in one
+// level: 32 lanes x 32 bytes, in two planes of 16-byte records,
+//   [0, 512)     lane l: 4 values (float4)
+//   [512, 1024)  lane l: 4 dependency slots (uint16), the row's own slot
+//                (uint16), flags (uint16), the factor the row's sum is
+//                multiplied by (float: 1 / u_ii, or 1)
+// A row of c <= 128 entries takes G = 1, 2, .. 32 lanes (the power of two at
+// or above c / 4), aligned to G; entry j + k G is value k of its lane j.
+// Flags: bits 0-2 log2 G, bits 3-5 the largest log2 G of the unit, bit 6 the
+// row's first lane (it holds the right-hand side and stores the result), bits
+// 7-12 the level barriers the warp passes before this unit, bit 13: one more
+// right after it (its next unit lies in a later level), before that unit is
+// loaded.
+constexpr int kLongWarps = 16;      // solving warps: unit u of a block is warp u mod 16's
+constexpr int kLongUnit = 1024;     // bytes of a unit
+constexpr int kLongPerLane = 4;     // entries per lane
+constexpr int kLongSlots = 65535;   // a block has fewer rows than this
 // The first violation a debug build (HEC_DEBUG) recorded: code, program,
 // chunk, thread, value, bound, 0, 0 (all 0: none); clear resets it.
 int trsv_debug_read(int *out, bool clear);
@@ -247,6 +266,8 @@ struct FillArgs {
     const int64_t *chunk_row0;
     const int *rm_start, *rm_len, *rm_diag; // factor entry of the pass's first value, count, diagonal
     const double *f;
+    int long_rows;           // 1: units of the long-row kernel; the maps have an entry per
+                             // lane: first entry, count | stride << 8, diagonal or -1
 };
 int launch_scatter_hec(int64_t nnz, const double *val, const int64_t *slot, double *ell,
                        double *tail, cudaStream_t s);

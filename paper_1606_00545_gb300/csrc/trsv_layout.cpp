@@ -837,6 +837,179 @@ void emit_resident(const BlockFactor &B, int FW, int vb, int NW, ResOut &O)
     O.largest = (size_t)O.group * cbytes;
 }
 
+// ------------------------------------------------------------------ long-row format
+// (k_trsv_long: units of kernels.cuh.)  The rows of a level, longest first,
+// are laid side by side in units; unit u of the block goes to warp u mod
+// kLongWarps, and kLongWarps consecutive units are one bulk copy.  Rows of
+// more than 32 x kLongPerLane entries take several pseudo-levels, each
+// subtracting its part of the sum.  L rows without entries need no work (y = r
+// is already in place).
+struct LongOut {
+    std::vector<unsigned char> bytes;
+    int units = 0, levels = 0, nL = 0, nU = 0, own0 = 0, own1 = 0;
+    std::vector<int> rm_start, rm_len, rm_diag; // per lane
+    int64_t alg = 0;
+};
+
+void emit_long(const BlockFactor &B, LongOut &O)
+{
+    const HostCSR &F = B.F;
+    const int nv = F.n, vb = 4;
+    BlockPlan bp;
+    needed_rows(B, bp);
+    bp.part.assign(nv, 0);
+    bp.posL.assign(nv, -1);
+    bp.posU.assign(nv, -1);
+    PassOrder po[2];
+    order_pass(B, bp, 0, false, po[0], bp.posL);
+    order_pass(B, bp, 0, true, po[1], bp.posU);
+    O.nL = (int)po[0].order.size();
+    O.nU = (int)po[1].order.size();
+    O.own0 = (int)(std::lower_bound(B.rows.begin(), B.rows.end(), B.own_lo) - B.rows.begin());
+    O.own1 = (int)(std::lower_bound(B.rows.begin(), B.rows.end(), B.own_hi) - B.rows.begin());
+    constexpr int kMost = kWarpRows * kLongPerLane;
+    struct Piece {
+        int row, e0, cnt, diag; // diag: the factor's entry index, -1: multiply by 1
+    };
+    // per warp: the level barriers it has passed, its last unit's level and place
+    std::vector<int> passed(kLongWarps, 0), last_level(kLongWarps, -1);
+    std::vector<size_t> last_off(kLongWarps, 0);
+    // the barrier of the warp's last unit's level, before a unit of level `l`
+    auto close_last = [&](int w, int l) {
+        if (last_level[w] < 0 || last_level[w] >= l)
+            return;
+        unsigned char *rec = O.bytes.data() + last_off[w] + 512;
+        for (int q = 0; q < kWarpRows; ++q)
+            reinterpret_cast<uint16_t *>(rec + 16 * q)[5] |= 1u << 13;
+        passed[w] = last_level[w] + 1;
+        last_level[w] = -1;
+    };
+    std::vector<Piece> ps;
+    auto emit_level = [&]() {
+        if (ps.empty())
+            return;
+        size_t i = 0;
+        while (i < ps.size()) { // one unit
+            const int u = O.units++;
+            const size_t off = O.bytes.size();
+            O.bytes.resize(off + kLongUnit, 0);
+            const size_t m0 = O.rm_start.size();
+            O.rm_start.resize(m0 + kWarpRows, 0);
+            O.rm_len.resize(m0 + kWarpRows, 0);
+            O.rm_diag.resize(m0 + kWarpRows, -1);
+            float *val = reinterpret_cast<float *>(O.bytes.data() + off);
+            unsigned char *rec = O.bytes.data() + off + 512;
+            int lane = 0, maxlg = 0;
+            uint16_t flags[kWarpRows] = {};
+            for (int l = 0; l < kWarpRows; ++l) { // idle lanes: padding slots, nothing stored
+                uint16_t *s = reinterpret_cast<uint16_t *>(rec + 16 * l);
+                for (int k = 0; k < kLongPerLane + 1; ++k)
+                    s[k] = (uint16_t)nv;
+                reinterpret_cast<float *>(rec + 16 * l)[3] = 1.0f;
+            }
+            while (i < ps.size()) {
+                const Piece &p = ps[i];
+                int lg = 0;
+                while ((kLongPerLane << lg) < p.cnt)
+                    ++lg;
+                const int G = 1 << lg;
+                if (lane + G > kWarpRows)
+                    break; // (pieces come longest first: lane is a multiple of G)
+                maxlg = std::max(maxlg, lg);
+                for (int j = 0; j < G; ++j, ++lane) {
+                    uint16_t *s = reinterpret_cast<uint16_t *>(rec + 16 * lane);
+                    int cnt = 0;
+                    for (int k = 0; k < kLongPerLane; ++k) {
+                        const int q = j + k * G;
+                        if (q >= p.cnt)
+                            break;
+                        val[lane * kLongPerLane + k] = (float)F.va[p.e0 + q];
+                        s[k] = (uint16_t)F.ci[p.e0 + q];
+                        ++cnt;
+                    }
+                    s[kLongPerLane] = (uint16_t)p.row;
+                    flags[lane] = (uint16_t)(lg | (j == 0 ? 64 : 0));
+                    const bool d = j == 0 && p.diag >= 0;
+                    if (d)
+                        reinterpret_cast<float *>(rec + 16 * lane)[3] = (float)(1.0 / F.va[p.diag]);
+                    O.rm_start[m0 + lane] = p.e0 + j;
+                    O.rm_len[m0 + lane] = cnt | (G << 8);
+                    O.rm_diag[m0 + lane] = d ? p.diag : -1;
+                }
+                ++i;
+            }
+            const int w = u % kLongWarps;
+            close_last(w, O.levels);
+            const int nbar = O.levels - passed[w];
+            passed[w] = O.levels;
+            last_level[w] = O.levels;
+            last_off[w] = off;
+            rec = O.bytes.data() + off + 512;
+            for (int l = 0; l < kWarpRows; ++l)
+                reinterpret_cast<uint16_t *>(rec + 16 * l)[5] =
+                    (uint16_t)(flags[l] | (maxlg << 3) | (nbar << 7));
+        }
+        ++O.levels;
+        ps.clear();
+    };
+    for (int pass = 0; pass < 2; ++pass) {
+        const bool upass = pass == 1;
+        int start = 0;
+        for (int end : po[pass].level_end) {
+            for (int q = start; q < end; ++q) {
+                const int i = po[pass].order[q], len = row_len(B, upass, i);
+                if (upass)
+                    O.alg += (4ll + vb) * len + 2 * vb + 8 + (bp.owned[i] ? vb : 0);
+                else
+                    O.alg += (4ll + vb) * len + 2 * vb + 4;
+            }
+            // rows are sorted longest first; part r of the level: entries
+            // [r kMost, ..) of the rows that have them
+            for (int r = 0;; ++r) {
+                bool more = false;
+                for (int q = start; q < end; ++q) {
+                    const int i = po[pass].order[q], len = row_len(B, upass, i);
+                    const int left = len - r * kMost;
+                    if (r > 0 ? left <= 0 : (!upass && len == 0))
+                        continue;
+                    const bool last = left <= kMost;
+                    more |= !last;
+                    ps.push_back({i, row_first(B, upass, i) + r * kMost, std::min(left, kMost),
+                                  upass && last ? B.diag[i] : -1});
+                }
+                // (rows of the same part differ in length: longest first again)
+                std::stable_sort(ps.begin(), ps.end(),
+                                 [](const Piece &x, const Piece &y) { return x.cnt > y.cnt; });
+                emit_level();
+                if (!more)
+                    break;
+            }
+            start = end;
+        }
+    }
+    for (int w = 0; w < kLongWarps; ++w)
+        close_last(w, O.levels);
+    // whole groups of kLongWarps units: the last ones idle
+    while (O.units % kLongWarps != 0) {
+        const int w = O.units % kLongWarps;
+        const size_t off = O.bytes.size();
+        O.bytes.resize(off + kLongUnit, 0);
+        O.rm_start.resize(O.rm_start.size() + kWarpRows, 0);
+        O.rm_len.resize(O.rm_len.size() + kWarpRows, 0);
+        O.rm_diag.resize(O.rm_diag.size() + kWarpRows, -1);
+        unsigned char *rec = O.bytes.data() + off + 512;
+        for (int l = 0; l < kWarpRows; ++l) {
+            uint16_t *s = reinterpret_cast<uint16_t *>(rec + 16 * l);
+            for (int k = 0; k < kLongPerLane + 1; ++k)
+                s[k] = (uint16_t)nv;
+            s[5] = (uint16_t)((O.levels - passed[w]) << 7);
+            reinterpret_cast<float *>(rec + 16 * l)[3] = 1.0f;
+        }
+        passed[w] = O.levels;
+        ++O.units;
+    }
+}
+
 } // namespace
 
 int trsv_resident_width(int longest_row)
@@ -929,6 +1102,70 @@ int pack_trsv_resident(const std::vector<BlockFactor> &Bs, int width, int vb, Tr
         P.alg_bytes += O.alg;
     }
     P.chunk_row0.push_back(r0);
+    return HEC_OK;
+}
+
+int pack_trsv_long(const std::vector<BlockFactor> &Bs, TrsvPack &P, std::string &msg)
+{
+    const int nb = (int)Bs.size();
+    for (const BlockFactor &B : Bs)
+        if (B.F.n >= kLongSlots) {
+            msg = "long-row layout: a block has 65535 rows or more";
+            return HEC_ERR_INVALID;
+        }
+    std::vector<LongOut> outs(nb);
+    parallel_for(nb, [&](int b) { emit_long(Bs[b], outs[b]); });
+    P = TrsvPack();
+    P.resident = 2;
+    P.parts = 1;
+    P.ring_slots = 32;
+    P.stage_bytes = kLongWarps * kLongUnit;
+    size_t total = 0;
+    for (const LongOut &O : outs)
+        total += O.bytes.size();
+    if (total / 16 > 0xffffffffull) {
+        msg = "factor layout exceeds 64 GiB";
+        return HEC_ERR_INVALID;
+    }
+    P.pack.resize(total);
+    P.blocks.assign(nb, TrsvBlock());
+    int64_t ent0 = 0;
+    size_t off = 0;
+    for (int b = 0; b < nb; ++b) {
+        const LongOut &O = outs[b];
+        TrsvBlock &T = P.blocks[b];
+        T.chunk_begin = T.chunk_mid = (int)P.chunks.size();
+        T.zoff = (int64_t)P.groups.size();
+        for (int u = 0; u < O.units; ++u) {
+            P.chunk_row0.push_back((int64_t)P.rm_start.size() + (int64_t)u * kWarpRows);
+            const unsigned o16 = (unsigned)((off + (size_t)u * kLongUnit) / 16);
+            P.chunks.push_back(make_uint2(o16, (unsigned)kLongUnit));
+            if (u % kLongWarps == 0)
+                P.groups.push_back(make_uint2(o16, (unsigned)(kLongWarps * kLongUnit)));
+        }
+        T.chunk_end = (int)P.chunks.size();
+        T.ngroups = O.units / kLongWarps;
+        T.ring_L = O.levels; // level barriers of the block
+        T.ring_U = 1;
+        T.yoff = (int64_t)P.vrows.size();
+        T.nv = Bs[b].F.n;
+        T.own0 = O.own0;
+        T.own1 = O.own1;
+        P.vrows.insert(P.vrows.end(), Bs[b].rows.begin(), Bs[b].rows.end());
+        P.res_slots = std::max(P.res_slots, T.nv + 1);
+        P.rows_L += O.nL;
+        P.rows_U += O.nU;
+        for (size_t k = 0; k < O.rm_start.size(); ++k) {
+            P.rm_start.push_back((int)(ent0 + O.rm_start[k]));
+            P.rm_len.push_back(O.rm_len[k]);
+            P.rm_diag.push_back(O.rm_diag[k] < 0 ? -1 : (int)(ent0 + O.rm_diag[k]));
+        }
+        ent0 += (int64_t)Bs[b].F.ci.size();
+        std::memcpy(P.pack.data() + off, O.bytes.data(), O.bytes.size());
+        off += O.bytes.size();
+        P.alg_bytes += O.alg;
+    }
+    P.chunk_row0.push_back((int64_t)P.rm_start.size());
     return HEC_OK;
 }
 
