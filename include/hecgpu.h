@@ -435,7 +435,7 @@ void hec_precond_destroy(hec_precond_t M);
  * host's operation order and rounding (the factors are bit-identical to a
  * fresh ilu_k_setup of the new matrix), and refills the values of its
  * triangular-solve layouts.  Solve graphs and handles stay valid.  The first
- * call per handle uploads index maps (about 12 bytes per matrix entry and 16
+ * call per handle uploads index maps (about 12 bytes per matrix entry and 20
  * per factor entry), later calls only stream values.  The call synchronises
  * the stream.  Returns HEC_OK, HEC_ERR_ZERO_PIVOT (the factors are then
  * unusable until the next successful refactor) or HEC_ERR_INVALID. */

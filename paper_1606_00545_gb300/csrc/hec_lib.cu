@@ -202,8 +202,9 @@ struct hec_precond_s {
     // hec_refactor: every block's factor on the device (entries numbered over
     // all blocks), its source map into A and the L level sets; the host copy
     // of the factor values is refreshed on demand
-    DevBuf rf_rp, rf_ci, rf_dg, rf_f, rf_src, rf_row0, rf_lev0, rf_lptr, rf_lrows;
+    DevBuf rf_rp, rf_ci, rf_dg, rf_f, rf_src, rf_row0, rf_lev0, rf_lptr, rf_lrows, rf_plan;
     int64_t rf_nent = 0;
+    int rf_longest = 0, rf_level_rows = 0; // longest factor row; mean rows of an L level (largest block)
     bool rf_ready = false, factor_host_stale = false;
     int64_t device_bytes() const
     {
@@ -211,7 +212,7 @@ struct hec_precond_s {
                (int64_t)dinv.bytes + (int64_t)dinv32.bytes + (int64_t)rf_rp.bytes +
                (int64_t)rf_ci.bytes + (int64_t)rf_dg.bytes + (int64_t)rf_f.bytes +
                (int64_t)rf_src.bytes + (int64_t)rf_row0.bytes + (int64_t)rf_lev0.bytes +
-               (int64_t)rf_lptr.bytes + (int64_t)rf_lrows.bytes;
+               (int64_t)rf_lptr.bytes + (int64_t)rf_lrows.bytes + (int64_t)rf_plan.bytes;
     }
     ~hec_precond_s();
 };
@@ -1265,6 +1266,26 @@ int refactor_matrix(hec_matrix_s *A, const double *val, cudaStream_t s)
     return HEC_OK;
 }
 
+RefactorArgs refactor_args(const hec_precond_s *M)
+{
+    RefactorArgs ra{};
+    ra.nent = M->rf_nent;
+    ra.src = M->rf_src.as<int>();
+    ra.f = M->rf_f.as<double>();
+    ra.rp = M->rf_rp.as<int>();
+    ra.ci = M->rf_ci.as<int>();
+    ra.dg = M->rf_dg.as<int>();
+    ra.blk_row0 = M->rf_row0.as<int>();
+    ra.blk_lev0 = M->rf_lev0.as<int>();
+    ra.lptr = M->rf_lptr.as<int>();
+    ra.lrows = M->rf_lrows.as<int>();
+    ra.err = M->d_err.as<int>();
+    ra.plan = M->rf_plan.as<uint32_t>();
+    ra.longest_row = M->rf_longest;
+    ra.level_rows = M->rf_level_rows;
+    return ra;
+}
+
 // The factor data of every block on the device, built on the first refactor.
 int upload_refactor_data(const hec_matrix_s *A, hec_precond_s *M, cudaStream_t s)
 {
@@ -1277,6 +1298,10 @@ int upload_refactor_data(const hec_matrix_s *A, hec_precond_s *M, cudaStream_t s
         row0[b + 1] = row0[b] + M->blocks[b].F.n;
         lev0[b + 1] = lev0[b] + (int)M->blocks[b].lptrL.size();
         nent += (int64_t)M->blocks[b].F.ci.size();
+        const HostCSR &F = M->blocks[b].F;
+        for (int i = 0; i < F.n; ++i)
+            M->rf_longest = std::max(M->rf_longest, F.rp[i + 1] - F.rp[i]);
+        M->rf_level_rows = std::max(M->rf_level_rows, F.n / std::max(1, M->blocks[b].nlevL));
     }
     if (nent >= INT32_MAX)
         return fail(HEC_ERR_INVALID, "factors of %lld entries exceed the refactor index range",
@@ -1322,6 +1347,11 @@ int upload_refactor_data(const hec_matrix_s *A, hec_precond_s *M, cudaStream_t s
     HEC_TRY(upload(M->rf_lptr, lptr, s));
     HEC_TRY(upload(M->rf_lrows, lrows, s));
     HEC_TRY(M->rf_f.alloc(nent * sizeof(double), s));
+    if (M->rf_longest <= kPlannedRow) {
+        HEC_TRY(M->rf_plan.alloc(nent * sizeof(uint32_t), s));
+        launch_refactor_plan(refactor_args(M), nb, s);
+        HEC_TRY(check_launch("elimination plan"));
+    }
     HEC_CK(cudaStreamSynchronize(s));
     M->rf_nent = nent;
     M->rf_ready = true;
@@ -1346,20 +1376,10 @@ int refactor_precond(hec_matrix_s *A, hec_precond_s *M, cudaStream_t s)
         return check_launch("jacobi dinv");
     }
     HEC_TRY(upload_refactor_data(A, M, s));
-    RefactorArgs ra{};
-    ra.nent = M->rf_nent;
+    RefactorArgs ra = refactor_args(M);
     ra.val = dval;
-    ra.src = M->rf_src.as<int>();
-    ra.f = M->rf_f.as<double>();
-    ra.rp = M->rf_rp.as<int>();
-    ra.ci = M->rf_ci.as<int>();
-    ra.dg = M->rf_dg.as<int>();
-    ra.blk_row0 = M->rf_row0.as<int>();
-    ra.blk_lev0 = M->rf_lev0.as<int>();
-    ra.lptr = M->rf_lptr.as<int>();
-    ra.lrows = M->rf_lrows.as<int>();
-    ra.err = M->d_err.as<int>();
-    launch_refactor(ra, M->nblocks, s);
+    if (launch_refactor(ra, M->nblocks, device_sms(), s) != 0)
+        return fail(HEC_ERR_CUDA, "cannot configure the elimination kernel");
     HEC_TRY(check_launch("refactor"));
     for (int idx = 0; idx < 2; ++idx) {
         TrsvLayout &L = M->lay[idx];

@@ -12,6 +12,9 @@
 // for the j of row p's U part that row i holds -- with separately rounded
 // multiply and subtract (no contraction, as the host code is compiled), so
 // the factors are bit-identical to a host factorisation of the new matrix.
+#include <mutex>
+
+#include "ptx.cuh"
 #include "reduce.cuh"
 
 namespace hec {
@@ -159,6 +162,171 @@ __global__ void __launch_bounds__(kThreads) k_iluk_numeric(RefactorArgs a)
     }
 }
 
+// The same elimination for blocks whose rows hold at most LEN entries.  The
+// merges of k_iluk_numeric chase one pivot entry at a time through memory,
+// and that latency, not the arithmetic, is its time (23 us a level on the
+// 101^3 ILU(1) case).  Here a row's values are in shared memory, a pivot's U
+// part comes in with independent loads, up to kAhead entries at once and one
+// pivot ahead of their use (the pivot's place in memory two ahead), and where
+// an entry goes is known from a plan made once per pattern (k_iluk_plan: 4
+// bits for each of those entries, 0 for none -- an update never hits position
+// 0); rows of 17 to 32 entries compare columns instead, which costs 2,000
+// instructions a row (4.8 ms on that case instead of 3.7).  What is left is the chain
+// of one division and a few updates per pivot.  A block's rows go to C CTAs
+// of a cluster, warp by warp, with a cluster barrier between levels: 64 blocks
+// alone leave most SMs idle.  101^3, ILU(1), 64 blocks: 7.08 -> 3.7 ms (of
+// hec_refactor's 8.2 -> 4.8 with an SpMV and an apply behind it).
+constexpr int kAhead = 8;
+
+// The position among the row's columns of column c, -1 if it holds none.
+template <int LEN> __device__ __forceinline__ int find_col(const int (&col)[LEN], int c)
+{
+    int x = -1;
+#pragma unroll
+    for (int j = 0; j < LEN; ++j)
+        x = col[j] == c ? j : x;
+    return x;
+}
+
+template <int LEN> __global__ void __launch_bounds__(kThreads) k_iluk_plan(RefactorArgs a)
+{
+    static_assert(LEN <= 16 && kAhead * 4 <= 32, "4 bits per entry");
+    const int row0 = a.blk_row0[blockIdx.x], nv = a.blk_row0[blockIdx.x + 1] - row0;
+    for (int i = blockIdx.y * kThreads + threadIdx.x; i < nv; i += gridDim.y * kThreads) {
+        const int r = row0 + i, b0 = a.rp[r], len = a.rp[r + 1] - b0, nl = a.dg[r] - b0;
+        int col[LEN];
+#pragma unroll
+        for (int x = 0; x < LEN; ++x)
+            col[x] = x < len ? a.ci[b0 + x] : 0x7fffffff;
+        for (int k = 0; k < nl; ++k) {
+            const int p = row0 + a.ci[b0 + k], y0 = a.dg[p] + 1, ep = a.rp[p + 1];
+            uint32_t plan = 0;
+#pragma unroll
+            for (int y = 0; y < kAhead; ++y)
+                if (y0 + y < ep) {
+                    const int x = find_col<LEN>(col, a.ci[y0 + y]);
+                    plan |= x > 0 ? (uint32_t)x << (4 * y) : 0u;
+                }
+            a.plan[b0 + k] = plan;
+        }
+    }
+}
+
+template <int LEN, bool PLAN>
+__global__ void __launch_bounds__(kThreads) k_iluk_rows(RefactorArgs a, int C)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    double *fs = reinterpret_cast<double *>(smem);            // [LEN][kThreads]
+    int *cs = reinterpret_cast<int *>(fs + LEN * kThreads);    // [LEN][kThreads]
+    const int t = threadIdx.x;
+    const int b = blockIdx.x / C, rank = blockIdx.x % C;
+    const int row0 = a.blk_row0[b];
+    const int *lptr = a.lptr + a.blk_lev0[b];
+    const int nlev = a.blk_lev0[b + 1] - a.blk_lev0[b] - 1;
+    const int *lrows = a.lrows + row0;
+    const int vt = ((t / 32) * C + rank) * 32 + t % 32; // warps in turn over the CTAs
+    for (int l = 0; l < nlev; ++l) {
+        const int q1 = lptr[l + 1];
+        for (int q = lptr[l] + vt; q < q1; q += kThreads * C) {
+            const int r = row0 + __ldg(&lrows[q]);
+            const int b0 = __ldg(&a.rp[r]), len = __ldg(&a.rp[r + 1]) - b0,
+                      nl = __ldg(&a.dg[r]) - b0;
+            int col[LEN];
+#pragma unroll
+            for (int x = 0; x < LEN; ++x)
+                col[x] = x < len ? __ldg(&a.ci[b0 + x]) : 0x7fffffff;
+#pragma unroll
+            for (int x = 0; x < LEN; ++x) {
+                cs[x * kThreads + t] = col[x];
+                if (x < len)
+                    fs[x * kThreads + t] = __ldcg(&a.f[b0 + x]);
+            }
+            // pivot k: its diagonal's and its row's end in memory and its plan;
+            // its U part
+            struct Place {
+                int dp, ep;
+                uint32_t plan;
+            };
+            struct Pivot {
+                double upp, u[kAhead];
+                int c[PLAN ? 1 : kAhead];
+            };
+            auto place = [&](int k) -> Place {
+                if (k >= nl)
+                    return Place{0, 0, 0u};
+                const int p = row0 + cs[k * kThreads + t];
+                return Place{__ldg(&a.dg[p]), __ldg(&a.rp[p + 1]),
+                             PLAN ? __ldg(&a.plan[b0 + k]) : 0u};
+            };
+            auto load = [&](const Place &pl, int k, Pivot &P) {
+                if (k >= nl)
+                    return;
+                P.upp = __ldcg(&a.f[pl.dp]);
+#pragma unroll
+                for (int y = 0; y < kAhead; ++y)
+                    if (PLAN ? (pl.plan >> (4 * y) & 15u) != 0u : pl.dp + 1 + y < pl.ep) {
+                        if constexpr (!PLAN)
+                            P.c[y] = __ldg(&a.ci[pl.dp + 1 + y]);
+                        P.u[y] = __ldcg(&a.f[pl.dp + 1 + y]);
+                    }
+            };
+            Place p0 = place(0), p1 = place(1);
+            Pivot P0, P1;
+            load(p0, 0, P0);
+            bool ok = true;
+            for (int k = 0; k < nl; ++k) {
+                const Place p2 = place(k + 2);
+                load(p1, k + 1, P1);
+                if (P0.upp == 0.0) {
+                    ok = false;
+                    break;
+                }
+                const double lip = __ddiv_rn(fs[k * kThreads + t], P0.upp);
+                fs[k * kThreads + t] = lip;
+                // the entries' columns differ, so their positions do: every
+                // load comes before the first store
+                int at[kAhead];
+                double g[kAhead];
+#pragma unroll
+                for (int y = 0; y < kAhead; ++y) {
+                    if constexpr (PLAN)
+                        at[y] = (int)(p0.plan >> (4 * y) & 15u);
+                    else
+                        at[y] = p0.dp + 1 + y < p0.ep ? find_col<LEN>(col, P0.c[y]) : -1;
+                }
+#pragma unroll
+                for (int y = 0; y < kAhead; ++y)
+                    if (at[y] > 0)
+                        g[y] = fs[at[y] * kThreads + t];
+#pragma unroll
+                for (int y = 0; y < kAhead; ++y)
+                    if (at[y] > 0)
+                        fs[at[y] * kThreads + t] = __dsub_rn(g[y], __dmul_rn(lip, P0.u[y]));
+                for (int e = p0.dp + 1 + kAhead; e < p0.ep; ++e) {
+                    const int x = find_col<LEN>(col, __ldg(&a.ci[e]));
+                    if (x > 0)
+                        fs[x * kThreads + t] =
+                            __dsub_rn(fs[x * kThreads + t], __dmul_rn(lip, __ldcg(&a.f[e])));
+                }
+                p0 = p1;
+                p1 = p2;
+                P0 = P1;
+            }
+#pragma unroll
+            for (int x = 0; x < LEN; ++x)
+                if (x < len)
+                    a.f[b0 + x] = fs[x * kThreads + t];
+            if (!ok || fs[nl * kThreads + t] == 0.0)
+                atomicExch(a.err, HEC_ERR_ZERO_PIVOT);
+        }
+        __syncwarp();
+        if (C > 1)
+            cluster_sync_all();
+        else
+            __syncthreads();
+    }
+}
+
 // The triangular-solve layout's value slots from the new factor values: one
 // CTA per chunk, thread t on row t.  Row t of chunk c takes the factor
 // entries [start, start + len) of its pass (L: the multipliers; U: the
@@ -263,11 +431,52 @@ int launch_cast_f32(int64_t n, const double *x, float *y, cudaStream_t s)
     return 0;
 }
 
-int launch_refactor(const RefactorArgs &a, int nblocks, cudaStream_t s)
+template <int LEN, bool PLAN>
+static int launch_rows(const RefactorArgs &a, int nblocks, int C, cudaStream_t s)
+{
+    constexpr int smem = LEN * kThreads * (int)(sizeof(double) + sizeof(int));
+    static std::once_flag once;
+    static cudaError_t e = cudaSuccess;
+    std::call_once(once, []() {
+        e = cudaFuncSetAttribute(k_iluk_rows<LEN, PLAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    });
+    if (e != cudaSuccess)
+        return -1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(nblocks * C));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k_iluk_rows<LEN, PLAN>, a, C) == cudaSuccess ? 0 : -1;
+}
+
+int launch_refactor_plan(const RefactorArgs &a, int nblocks, cudaStream_t s)
+{
+    k_iluk_plan<kPlannedRow><<<dim3(nblocks, std::max(1, 8192 / nblocks)), kThreads, 0, s>>>(a);
+    return 0;
+}
+
+int launch_refactor(const RefactorArgs &a, int nblocks, int sms, cudaStream_t s)
 {
     k_gather_factor<<<grid_of(a.nent), 256, 0, s>>>(a.nent, a.val, a.src, a.f);
-    k_iluk_numeric<<<nblocks, kThreads, 0, s>>>(a);
-    return 0;
+    if (a.longest_row > 32) { // longer rows do not fit the registers and shared memory
+        k_iluk_numeric<<<nblocks, kThreads, 0, s>>>(a);
+        return 0;
+    }
+    // CTAs per block: while the SMs allow it and a level keeps every CTA at
+    // least a warp of rows
+    int C = 1;
+    while (C < 8 && 2 * C * nblocks <= sms && a.level_rows >= 2 * C * 32)
+        C *= 2;
+    return a.longest_row <= kPlannedRow ? launch_rows<kPlannedRow, true>(a, nblocks, C, s)
+                                        : launch_rows<32, false>(a, nblocks, C, s);
 }
 
 int launch_fill_pack(const FillArgs &a, int nchunks, bool fp32, cudaStream_t s)

@@ -258,6 +258,10 @@ struct RefactorArgs {
     const int *blk_lev0;     // nblocks + 1: offsets into lptr (each block: nlev + 1 entries)
     const int *lptr, *lrows; // L level sets per block (local rows, by block row offset)
     int *err;                // device error word (HEC_ERR_ZERO_PIVOT)
+    uint32_t *plan;          // per factor entry of L: where its pivot's entries go (k_iluk_plan;
+                             // rows of at most kPlannedRow entries)
+    int longest_row;         // entries of the longest factor row
+    int level_rows;          // mean rows of an L level, of the block where it is largest
 };
 // Per row of every chunk of a triangular-solve layout: where its values come from.
 struct FillArgs {
@@ -272,7 +276,9 @@ struct FillArgs {
 int launch_scatter_hec(int64_t nnz, const double *val, const int64_t *slot, double *ell,
                        double *tail, cudaStream_t s);
 int launch_cast_f32(int64_t n, const double *x, float *y, cudaStream_t s);
-int launch_refactor(const RefactorArgs &a, int nblocks, cudaStream_t s);
+constexpr int kPlannedRow = 16;
+int launch_refactor_plan(const RefactorArgs &a, int nblocks, cudaStream_t s); // once per pattern
+int launch_refactor(const RefactorArgs &a, int nblocks, int sms, cudaStream_t s);
 int launch_fill_pack(const FillArgs &a, int nchunks, bool fp32, cudaStream_t s);
 int launch_jacobi_dinv(int n, const double *val, const int64_t *diag, double omega, double *dinv,
                        float *dinv32, int *err, cudaStream_t s);
