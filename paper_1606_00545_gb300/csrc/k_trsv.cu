@@ -345,22 +345,19 @@ template <class T, int FW> struct RowRegs {
     __device__ int d(int k) const { return get4(dv[k / 4], k % 4); }
 };
 
-// Row t = 32 w + lane of a chunk.  Warps past the chunk's last one read the
-// header only; past it, every address depends on the stage, the thread and
-// the pass alone: all loads issue back to back, 16 bytes each for the row's
-// entries.
+// Row t = 32 w + lane of a chunk (header hdr).  Every address depends on the
+// stage, the thread and the pass alone: all loads issue back to back, 16
+// bytes each for the row's entries.
 template <class T, int FW>
-__device__ __forceinline__ void load_fixed(const unsigned char *ch, const T *rslot, int w, int lane,
-                                           bool upass, bool exps, RowRegs<T, FW> &R)
+__device__ __forceinline__ void load_fixed(const unsigned char *ch, const int4 &hdr, const T *rslot,
+                                           int w, int lane, bool upass, bool exps,
+                                           RowRegs<T, FW> &R)
 {
     using F = Fixed<T, FW>;
-    const int4 hdr = *reinterpret_cast<const int4 *>(ch);
     R.nrows = hdr.x;
     R.nwarps = hdr.y;
     R.base = hdr.z;
     R.flags = hdr.w;
-    if (w >= hdr.y)
-        return;
     const unsigned char *blk = ch + kFixedHeader + (size_t)w * F::block(upass, exps);
     const typename Vec16<T>::type *val = reinterpret_cast<const typename Vec16<T>::type *>(blk) + lane;
 #pragma unroll
@@ -438,9 +435,8 @@ __device__ __forceinline__ bool issue_chunks(const uint2 *chunks, int nch, int S
 //             and a barrier of both ends every level.  While one set solves
 //             chunk c -- ring loads, the row's multiply-add chain, the result
 //             into the ring (for exports also into the neighbour's import
-//             ring) -- the other confirms that chunk c + 1 has been handed
-//             over, copies its rows into registers and forms every address
-//             its level will need.  So a level's critical path holds none of
+//             ring) -- the other copies chunk c + 1's rows into registers and
+//             forms every address its level will need.  So a level's critical path holds none of
 //             that: with one set doing all of it, the next chunk's copy and
 //             address arithmetic were the longer half of a level.  128^3,
 //             ILU(1), 64 blocks in two parts: FP64 apply 428 -> 330 us;
@@ -754,20 +750,53 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
             T *own = nullptr, *gout = nullptr;
             T acc = T(0);
             bool rows = false, mine = false, exports = false;
-            // copies this set's next chunk, c, in stage s, once it has been
-            // handed over, and forms every address its level will need
-            auto fetch = [&](int c) {
-                rows = mine = exports = false;
-                gout = nullptr;
+            // FP32, unsplit blocks: the set's last warp (with the shortest or
+            // no rows) confirms a chunk's handover a level before the set
+            // that copies it, so that the copy starts right after the barrier
+            // with the header in the first load, and the last result's global
+            // copy is written while the loads are under way: there the copy,
+            // not the chain, paces a level (128^3 280 -> 262 us, 101^3 242 ->
+            // 234).  In FP64 the chain does, and the same order costs (128^3
+            // 327 -> 340, 101^3 463 -> 471); in split blocks, asking a level
+            // early ties the parts closer together.
+            constexpr bool kAhead = sizeof(T) == 4;
+            const bool ahead = kAhead && !clustered;
+            const bool confirmer = ahead && w == kMaxWarps - 1;
+            auto confirm = [&](int st, uint32_t par) -> bool {
                 if (*vfail)
-                    return;
-                if (!handed(s, hpar)) {
-                    *vfail = 1;
-                    return;
+                    return false;
+                if (handed(st, par))
+                    return true;
+                *vfail = 1;
+                return false;
+            };
+            // copies this set's next chunk, c, in stage s, and forms every
+            // address the chunk's level will need
+            auto fetch = [&](int c) {
+                const unsigned char *ch = stages + (size_t)s * a.stage_bytes;
+                if (ahead) {
+                    const int fail = *vfail;
+                    const int4 hdr = *reinterpret_cast<const int4 *>(ch);
+                    rows = !fail && w < hdr.y; // warps past the chunk's last one hold no rows
+                    if (rows)
+                        load_fixed<T, FW>(ch, hdr, rhs + (size_t)s * kThreads, w, lane, U, exps,
+                                          R);
+                    if (gout)
+                        *gout = acc;
+                } else {
+                    if (gout)
+                        *gout = acc;
+                    rows = confirm(s, hpar);
+                    if (rows) {
+                        const int4 hdr = *reinterpret_cast<const int4 *>(ch);
+                        rows = w < hdr.y;
+                        if (rows)
+                            load_fixed<T, FW>(ch, hdr, rhs + (size_t)s * kThreads, w, lane, U,
+                                              exps, R);
+                    }
                 }
-                load_fixed<T, FW>(stages + (size_t)s * a.stage_bytes, rhs + (size_t)s * kThreads,
-                                  w, lane, U, exps, R);
-                rows = w < R.nwarps; // warps past the chunk's last one hold no rows
+                mine = exports = false;
+                gout = nullptr;
                 if (!rows)
                     return;
 #ifdef HEC_DEBUG
@@ -838,6 +867,13 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
                     hpar ^= 1u;
                 }
             };
+            // the confirmation of chunk n, the one after that in stage s
+            auto confirm_next = [&](int n) {
+                if (confirmer && n < c1) {
+                    const bool wrap = s + 1 == S;
+                    confirm(wrap ? 0 : s + 1, wrap ? hpar ^ 1u : hpar);
+                }
+            };
             // the stage of a chunk copied before the last barrier is free
             auto free_stage = [&](int c) {
                 if (row == 0 && c < c1)
@@ -848,6 +884,11 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
                 s_base = 0;
 #endif
             int c = c0 + set; // the chunk this set solves next, in stage s
+            if (set == 1)
+                advance();
+            if (confirmer && c < c1)
+                confirm(s, hpar);
+            solvers_sync<NT>();
             if (set == 0)
                 fetch(c);
             solvers_sync<NT>();
@@ -855,9 +896,10 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
                 free_stage(c);
                 advance();
             } else { // level c0 belongs to set 0
-                advance();
-                if (c < c1)
+                if (c < c1) {
                     fetch(c);
+                    confirm_next(c + 1);
+                }
                 solvers_sync<NT>();
                 free_stage(c);
                 advance();
@@ -876,18 +918,20 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
                 // ---- level c + 1: the other set solves, this one fetches
                 if (signal && row == 0)
                     st_release_cta_u32(&s_done, (uint32_t)(c + 1));
-                if (gout)
-                    *gout = acc;
                 if (c + 1 >= c1)
                     break;
                 advance();
-                if (c + 2 < c1)
+                if (c + 2 < c1) {
                     fetch(c + 2);
+                    confirm_next(c + 3);
+                }
                 solvers_sync<NT>();
                 free_stage(c + 2);
                 advance();
                 c += 2;
             }
+            if (gout) // the last result's global copy
+                *gout = acc;
         };
         auto pass = [&](auto Ucst, int c0, int c1) {
             constexpr bool U = decltype(Ucst)::value;
