@@ -1,6 +1,9 @@
 // k_vec.cu -- vector operations (Section 2.3, Eqs. 3-6) and the fused vector
 // updates of the Krylov loops (Algorithm 4 and GMRES), each with its dot
 // products reduced in the same launch.
+#include <mutex>
+
+#include "ptx.cuh"
 #include "reduce.cuh"
 
 namespace hec {
@@ -542,6 +545,201 @@ int launch_basis_combine(const BasisArgs &a, int grid, cudaStream_t s, bool fp32
     else
         k_basis_combine<double><<<grid, kThreads, 0, s>>>(a);
     return 0;
+}
+
+// ------------------------------------------------------------------ small systems
+// The Arnoldi step of a small system is bound by its launches and by the
+// reduction at the end of each, not by the vectors.  Here one cluster of kArnoldiCtas CTAs keeps w
+// in registers (a thread owns up to kArnoldiPerThread rows), and a reduction is
+// one exchange of per-CTA sums through distributed shared memory: every CTA
+// stores its sums into every other's, a cluster barrier, and all add them in
+// the same order.  16 CTAs: the FP64 unit is the SM's, so 8 would take the
+// multiply-adds twice as long.  The basis is read four times, the last three
+// from L1.  64^2 GMRES(30) solve: 11.8 -> 11.2 ms; what bounds it now is the
+// chain of FP64 adds (65 cycles each, one in flight per warp) of three
+// reductions and the Givens step.
+struct ArnoldiShared {
+    double part[3][kArnoldiCtas][kArnoldiRestart + 1]; // per exchange: each CTA's sums
+    double warp[kThreads / 32][kArnoldiRestart + 2];
+    double h[kArnoldiRestart + 1];
+};
+
+// Sums over the cluster of the cnt values that warp w of this CTA left in
+// S.warp[w][0 .. cnt), into S.h; exchange x of the launch.
+__device__ __forceinline__ void cluster_sums(ArnoldiShared &S, int x, int cnt, int rank)
+{
+    const int t = threadIdx.x;
+    __syncthreads();
+    if (t < cnt) {
+        double s = 0.0;
+#pragma unroll
+        for (int w = 0; w < kThreads / 32; ++w)
+            s += S.warp[w][t];
+        const uint32_t to = smem_u32(&S.part[x][rank][t]);
+        for (int c = 0; c < kArnoldiCtas; ++c)
+            st_cluster(mapa_shared(to, c), s);
+    }
+    cluster_sync_all();
+    for (int q0 = 0; q0 < cnt; q0 += kThreads / 8) { // eight lanes per value
+        const int q = q0 + t / 8, l = t % 8;
+        double s = q < cnt ? S.part[x][l][q] + S.part[x][l + 8][q] : 0.0;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (q < cnt && l == 0)
+            S.h[q] = s;
+    }
+    __syncthreads();
+}
+
+template <class T> __global__ void __launch_bounds__(kThreads) k_arnoldi(BasisArgs a)
+{
+    static_assert(kArnoldiCtas == 16, "cluster_sums adds two CTAs per lane");
+    __shared__ ArnoldiShared S;
+    count_launch(a.st);
+    SolverState *st = a.st;
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+    const int rank = (int)cluster_ctarank();
+    cluster_sync_all(); // every CTA runs before another one stores into it
+    const int j = st->j, k = j + 1;
+    const T *__restrict__ V = reinterpret_cast<const T *>(a.V);
+    const T *w_in = reinterpret_cast<const T *>(a.w);
+    constexpr int Q = kArnoldiPerThread, stride = kArnoldiCtas * kThreads;
+    const int i0 = rank * kThreads + t;
+    T w[Q];
+    T ww = T(0);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+        w[q] = i0 + q * stride < a.n ? w_in[i0 + q * stride] : T(0);
+        ww = fma(w[q], w[q], ww);
+    }
+    // warp sums of (V_g, w), g < k, into S.warp[wid]
+    auto project = [&]() {
+        for (int g0 = 0; g0 < k; g0 += kGroup) {
+            T acc[kGroup];
+#pragma unroll
+            for (int g = 0; g < kGroup; ++g)
+                acc[g] = T(0);
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (i0 + q * stride < a.n) {
+#pragma unroll
+                    for (int g = 0; g < kGroup; ++g)
+                        if (g0 + g < k)
+                            acc[g] = fma(__ldg(&V[(int64_t)(g0 + g) * a.ldv + i0 + q * stride]),
+                                         w[q], acc[g]);
+                }
+            double v[kGroup];
+#pragma unroll
+            for (int g = 0; g < kGroup; ++g)
+                v[g] = double(acc[g]);
+            const double s = warp_sum_group(v, lane);
+            const int g = g0 + ((lane >> 2) & 7);
+            if ((lane & 3) == 0 && g < k)
+                S.warp[wid][g] = s;
+        }
+    };
+    // w -= V h
+    auto subtract = [&]() {
+        for (int g0 = 0; g0 < k; g0 += kGroup)
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (i0 + q * stride < a.n) {
+                    T v[kGroup];
+#pragma unroll
+                    for (int g = 0; g < kGroup; ++g)
+                        if (g0 + g < k)
+                            v[g] = __ldg(&V[(int64_t)(g0 + g) * a.ldv + i0 + q * stride]);
+#pragma unroll
+                    for (int g = 0; g < kGroup; ++g)
+                        if (g0 + g < k)
+                            w[q] = fma(-T(S.h[g0 + g]), v[g], w[q]);
+                }
+    };
+    auto norm2 = [&]() {
+        T s = T(0);
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+            s = fma(w[q], w[q], s);
+        return s;
+    };
+    project();
+    const double ws = warp_sum(double(ww));
+    if (lane == 0)
+        S.warp[wid][k] = ws;
+    cluster_sums(S, 0, k + 1, rank); // h1, ||w||^2
+    if (rank == 0) {
+        if (t < k)
+            st->h1[t] = S.h[t];
+        if (t == 0)
+            st->w0norm = sqrt(S.h[k]);
+    }
+    subtract();
+    project();
+    cluster_sums(S, 1, k, rank); // h2
+    if (rank == 0 && t < k)
+        st->h2[t] = S.h[t];
+    subtract();
+    const double ns = warp_sum(double(norm2()));
+    __syncthreads(); // S.h and S.warp have been read
+    if (lane == 0)
+        S.warp[wid][0] = ns;
+    cluster_sums(S, 2, 1, rank);
+    const double nn = S.h[0];
+    // v_{j+1} (not read when the cycle ends here)
+    const double sc = 1.0 / sqrt(nn);
+    T *vn = reinterpret_cast<T *>(a.wout) + (int64_t)k * a.ldv;
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+        if (i0 + q * stride < a.n)
+            vn[i0 + q * stride] = T(sc * double(w[q]));
+    if (rank == 0)
+        finalize_gmres_step(&nn, st);
+}
+
+static cudaLaunchConfig_t arnoldi_config(cudaLaunchAttribute *attr, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kArnoldiCtas);
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = kArnoldiCtas;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+template <class T> static bool arnoldi_ready()
+{
+    // a cluster of 16 is above the portable size: allowed once per process
+    static std::once_flag once;
+    static bool ok = false;
+    std::call_once(once, []() {
+        cudaLaunchAttribute attr;
+        const cudaLaunchConfig_t cfg = arnoldi_config(&attr, nullptr);
+        int clusters = 0;
+        ok = cudaFuncSetAttribute(k_arnoldi<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                 cudaSuccess &&
+             cudaOccupancyMaxActiveClusters(&clusters, k_arnoldi<T>, &cfg) == cudaSuccess &&
+             clusters > 0;
+        if (!ok)
+            cudaGetLastError(); // the several-launch form runs instead
+    });
+    return ok;
+}
+
+bool arnoldi_available(bool fp32) { return fp32 ? arnoldi_ready<float>() : arnoldi_ready<double>(); }
+
+int launch_arnoldi(const BasisArgs &a, cudaStream_t s, bool fp32)
+{
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = arnoldi_config(&attr, s);
+    const cudaError_t e = fp32 ? cudaLaunchKernelEx(&cfg, k_arnoldi<float>, a)
+                               : cudaLaunchKernelEx(&cfg, k_arnoldi<double>, a);
+    return e == cudaSuccess ? 0 : -1;
 }
 
 // ------------------------------------------------------------------ small kernels

@@ -163,6 +163,16 @@ int launch_multidot(const BasisArgs &a, int sms, cudaStream_t s, bool fp32 = fal
 // wout = w - sum_i coef[i] V_i  (with_norm: + fused (wout, wout) -> op)
 int launch_basis_update(const BasisArgs &a, bool with_norm, int grid, cudaStream_t s,
                         bool fp32 = false);
+// One Arnoldi step after w = A z for small systems, as one cluster: ||w||, two
+// classical Gram-Schmidt projections of w against V_0 .. V_j (j = st->j),
+// h_{j+1,j}, the Givens update and V_{j+1} = w / h_{j+1,j}.  n at most
+// kArnoldiRows, restart at most kArnoldiRestart.
+constexpr int kArnoldiCtas = 16;
+constexpr int kArnoldiPerThread = 2;
+constexpr int kArnoldiRows = kArnoldiCtas * kThreads * kArnoldiPerThread;
+constexpr int kArnoldiRestart = 32;
+bool arnoldi_available(bool fp32); // the device can hold the cluster
+int launch_arnoldi(const BasisArgs &a, cudaStream_t s, bool fp32);
 // wout = sum_i coef[i] V_i
 int launch_basis_combine(const BasisArgs &a, int grid, cudaStream_t s, bool fp32 = false);
 
