@@ -102,7 +102,7 @@ __device__ __forceinline__ T warp_sum_t(T v)
 template <class T> constexpr int spmv_tiles_per_block() { return RowVec<T>::RPT / 2; }
 
 template <int MODE, int NDOT, bool TAIL, class T>
-__global__ void __launch_bounds__(kThreads, TAIL ? 1 : NDOT > 0 ? 6 : 8) k_spmv_hec(SpmvArgs a)
+__global__ void __launch_bounds__(kThreads, NDOT > 0 ? 6 : TAIL ? 0 : 8) k_spmv_hec(SpmvArgs a)
 {
     using RV = RowVec<T>;
     constexpr int RPT = RV::RPT, TPB = RPT / 2, BR = kThreads * RPT;
@@ -116,7 +116,9 @@ __global__ void __launch_bounds__(kThreads, TAIL ? 1 : NDOT > 0 ? 6 : 8) k_spmv_
     // and 4 per SM launched (see spmv_grid), the 128^3 SpMV with two dots
     // takes 46 us (61 before, 32 without dots; the FP64 pipe alone needs 30
     // for its 9 multiply-adds a row).  8 CTAs per SM spill: 47-51 us; the
-    // dots' partners loaded ahead of the slab: 56 us.
+    // dots' partners loaded ahead of the slab: 56 us.  Without dots 32
+    // registers, 8 CTAs per SM; left to itself the compiler takes 64 for the
+    // forms with tail rows (95^3 irregular 27-point, FP32: 47 us, 41 so).
     __shared__ T s_acc[NDOT > 0 ? NDOT : 1][NDOT > 0 ? kThreads : 1];
 #pragma unroll
     for (int d = 0; d < NDOT; ++d)
