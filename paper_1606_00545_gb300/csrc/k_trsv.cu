@@ -13,9 +13,9 @@
 // for U the destination row and the inverted diagonal, and for rows a
 // neighbouring part reads, the slot they go to there.  Two chunk formats:
 //   - fixed-slot (every row padded to one width FW <= 8): each thread's data
-//     sits at a compile-time offset from the stage, so the solving warps copy
-//     their rows of the next chunk into registers while the current chunk's
-//     multiply-add chain runs -- a level's critical path is then the ring
+//     sits at a compile-time offset from the stage, and one set of solving
+//     warps copies its rows of the next chunk into registers while the other
+//     set solves the current one -- a level's critical path is then the ring
 //     loads, the chain and the barrier;
 //   - generic (wider rows): per-warp widths, rows solved from shared memory.
 // Nothing on a level's critical path waits for HBM:
@@ -24,8 +24,8 @@
 //     on mbarriers, S chunks ahead of the solving warps;
 //   - four gatherer warps, taking chunks in turn, gather each landed chunk's
 //     right-hand sides (L pass: from r; U pass: from the L results, once the
-//     L pass is complete) with 4- or 8-byte cp.async, one chunk ahead, and
-//     hand the chunk over (a per-stage release-add counter) once the copies
+//     L pass is complete) with 4- or 8-byte cp.async, ahead of the solving
+//     warps, and hand the chunk over (an mbarrier per stage) once the copies
 //     have completed and the neighbouring parts have completed the chunks its
 //     thresholds name;
 //   - solved values of the last few levels live in a shared-memory ring
@@ -429,18 +429,19 @@ __device__ __forceinline__ bool issue_chunks(const uint2 *chunks, int nch, int S
 //             completed (waited for while the warp's next chunks are gathered)
 //             and lane 0 has seen the neighbouring parts' progress counters
 //             reach the chunk's thresholds, lane 0 arrives on the stage's
-//             handover mbarrier (a release-add to a shared counter instead
-//             waits for every copy of the warp still in flight);
+//             handover mbarrier (40 cycles; a release-add to a shared counter
+//             takes 90);
 //   solvers, fixed-slot chunks: two sets of 8 warps take the chunks in turn,
 //             and a barrier of both ends every level.  While one set solves
 //             chunk c -- ring loads, the row's multiply-add chain, the result
 //             into the ring (for exports also into the neighbour's import
 //             ring) -- the other copies chunk c + 1's rows into registers and
-//             forms every address its level will need.  So a level's critical path holds none of
-//             that: with one set doing all of it, the next chunk's copy and
-//             address arithmetic were the longer half of a level.  128^3,
-//             ILU(1), 64 blocks in two parts: FP64 apply 428 -> 330 us;
-//             101^3: 557 -> 463; 32^3, 8 blocks: 109 -> 78 (FP32 72 -> 52).
+//             forms every address its level will need.  So a level's
+//             critical path holds none of that: with one set doing all of it,
+//             the next chunk's copy and address arithmetic were the longer
+//             half of a level.  128^3, ILU(1), 64 blocks in two parts: FP64
+//             apply 427 -> 323 us; 101^3: 557 -> 457; 32^3, 8 blocks: 109 ->
+//             78 (FP32 72 -> 52).
 //             Three sets of 4 warps, with the addresses formed in a level of
 //             their own, were no faster (335 us), and adding the older
 //             levels' entries ahead of the barrier slower (410): the FP64
