@@ -22,7 +22,7 @@
 //   - an issuer warp streams chunks into a ring of shared-memory stages with
 //     cp.async.bulk (the TMA bulk-copy engine, evict-first in L2) completing
 //     on mbarriers, S chunks ahead of the solving warps;
-//   - four gatherer warps, taking chunks in turn, gather each landed chunk's
+//   - two gatherer warps, taking chunks in turn, gather each landed chunk's
 //     right-hand sides (L pass: from r; U pass: from the L results, once the
 //     L pass is complete) with 4- or 8-byte cp.async, ahead of the solving
 //     warps, and hand the chunk over (an mbarrier per stage) once the copies
@@ -62,10 +62,13 @@ size_t trsv_smem_bytes(int stage_bytes, int nstages, int ring_slots, int vbytes)
 // Gatherer warps of a CTA: they take the chunks in turn and keep up to
 // kGatherDepth chunks' right-hand-side gathers in flight each.  (Two, three
 // or four gatherers, depths 2 and 4: within 4% on the 128^3 case.)
-constexpr int kGatherers = 4;
+constexpr int kGatherers = 2;
 constexpr int kGatherDepth = 2;
 
 constexpr int kMaxStages = 16; // of the streamed kernel
+// Shared memory and (with two gatherer warps, 640 threads) registers left on
+// the SM for the vector and reduction kernels of other streams.
+constexpr int kLeaveFree = 24 * 1024;
 
 int trsv_stages_for(int stage_bytes, int ring_slots, int vbytes)
 {
@@ -73,7 +76,7 @@ int trsv_stages_for(int stage_bytes, int ring_slots, int vbytes)
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         optin = 227 * 1024;
-    optin -= 1024; // static shared memory of the kernel
+    optin -= kLeaveFree; // and its own static shared memory
     int S = kMaxStages;
     while (S > 3 && trsv_smem_bytes(stage_bytes, S, ring_slots, vbytes) > (size_t)optin)
         --S;
@@ -418,11 +421,11 @@ __device__ __forceinline__ bool issue_chunks(const uint2 *chunks, int nch, int S
 }
 
 // Warp-specialised CTA: 8 warps (fixed-slot chunks: two sets of 8) solve rows,
-// one row per thread per chunk; the last six warps feed them.  Per chunk c
+// one row per thread per chunk; the last four warps feed them.  Per chunk c
 // in stage s = c mod S:
 //   issuer: wait empty[s] (chunk c - S released) -> arm full[s] with
 //             the chunk's byte count -> cp.async.bulk the chunk;
-//   gatherers (four warps, chunks in turn): wait full[s] -> gather
+//   gatherers (two warps, chunks in turn): wait full[s] -> gather
 //             the chunk's right-hand sides into slot s with cp.async, one
 //             commit group per chunk (a U chunk waits for ldone first: its
 //             right-hand side is the L pass's output) -> once the group has

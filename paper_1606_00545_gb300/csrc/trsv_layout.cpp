@@ -871,6 +871,12 @@ void emit_long(const BlockFactor &B, LongOut &O)
     struct Piece {
         int row, e0, cnt, diag; // diag: the factor's entry index, -1: multiply by 1
     };
+    // about the entries at half-full lanes, and a unit for every narrow level
+    const size_t guess = F.ci.size() / 64 + po[0].level_end.size() + po[1].level_end.size() + 64;
+    O.bytes.reserve(guess * kLongUnit);
+    O.rm_start.reserve(guess * kWarpRows);
+    O.rm_len.reserve(guess * kWarpRows);
+    O.rm_diag.reserve(guess * kWarpRows);
     // per warp: the level barriers it has passed, its last unit's level and place
     std::vector<int> passed(kLongWarps, 0), last_level(kLongWarps, -1);
     std::vector<size_t> last_off(kLongWarps, 0);
@@ -1127,44 +1133,58 @@ int pack_trsv_long(const std::vector<BlockFactor> &Bs, TrsvPack &P, std::string 
         msg = "factor layout exceeds 64 GiB";
         return HEC_ERR_INVALID;
     }
-    P.pack.resize(total);
+    // where every block's units start (the row lists follow the blocks too)
+    std::vector<int64_t> unit0(nb + 1, 0), ent0(nb + 1, 0), row0(nb + 1, 0);
     P.blocks.assign(nb, TrsvBlock());
-    int64_t ent0 = 0;
-    size_t off = 0;
     for (int b = 0; b < nb; ++b) {
         const LongOut &O = outs[b];
+        unit0[b + 1] = unit0[b] + O.units;
+        ent0[b + 1] = ent0[b] + (int64_t)Bs[b].F.ci.size();
+        row0[b + 1] = row0[b] + Bs[b].F.n;
         TrsvBlock &T = P.blocks[b];
-        T.chunk_begin = T.chunk_mid = (int)P.chunks.size();
-        T.zoff = (int64_t)P.groups.size();
-        for (int u = 0; u < O.units; ++u) {
-            P.chunk_row0.push_back((int64_t)P.rm_start.size() + (int64_t)u * kWarpRows);
-            const unsigned o16 = (unsigned)((off + (size_t)u * kLongUnit) / 16);
-            P.chunks.push_back(make_uint2(o16, (unsigned)kLongUnit));
-            if (u % kLongWarps == 0)
-                P.groups.push_back(make_uint2(o16, (unsigned)(kLongWarps * kLongUnit)));
-        }
-        T.chunk_end = (int)P.chunks.size();
+        T.chunk_begin = T.chunk_mid = (int)unit0[b];
+        T.chunk_end = (int)unit0[b + 1];
+        T.zoff = unit0[b] / kLongWarps;
         T.ngroups = O.units / kLongWarps;
         T.ring_L = O.levels; // level barriers of the block
         T.ring_U = 1;
-        T.yoff = (int64_t)P.vrows.size();
+        T.yoff = row0[b];
         T.nv = Bs[b].F.n;
         T.own0 = O.own0;
         T.own1 = O.own1;
-        P.vrows.insert(P.vrows.end(), Bs[b].rows.begin(), Bs[b].rows.end());
         P.res_slots = std::max(P.res_slots, T.nv + 1);
         P.rows_L += O.nL;
         P.rows_U += O.nU;
-        for (size_t k = 0; k < O.rm_start.size(); ++k) {
-            P.rm_start.push_back((int)(ent0 + O.rm_start[k]));
-            P.rm_len.push_back(O.rm_len[k]);
-            P.rm_diag.push_back(O.rm_diag[k] < 0 ? -1 : (int)(ent0 + O.rm_diag[k]));
-        }
-        ent0 += (int64_t)Bs[b].F.ci.size();
-        std::memcpy(P.pack.data() + off, O.bytes.data(), O.bytes.size());
-        off += O.bytes.size();
         P.alg_bytes += O.alg;
     }
+    const size_t units = (size_t)unit0[nb];
+    P.pack.resize(total);
+    P.chunks.resize(units);
+    P.groups.resize(units / kLongWarps);
+    P.chunk_row0.resize(units);
+    P.vrows.resize((size_t)row0[nb]);
+    P.rm_start.resize(units * kWarpRows);
+    P.rm_len.resize(units * kWarpRows);
+    P.rm_diag.resize(units * kWarpRows);
+    parallel_for(nb, [&](int b) {
+        const LongOut &O = outs[b];
+        for (int u = 0; u < O.units; ++u) {
+            const int64_t g = unit0[b] + u;
+            const unsigned o16 = (unsigned)(g * kLongUnit / 16);
+            P.chunk_row0[g] = g * kWarpRows;
+            P.chunks[g] = make_uint2(o16, (unsigned)kLongUnit);
+            if (u % kLongWarps == 0)
+                P.groups[g / kLongWarps] = make_uint2(o16, (unsigned)(kLongWarps * kLongUnit));
+        }
+        const size_t m = (size_t)unit0[b] * kWarpRows;
+        for (size_t k = 0; k < O.rm_start.size(); ++k) {
+            P.rm_start[m + k] = (int)(ent0[b] + O.rm_start[k]);
+            P.rm_len[m + k] = O.rm_len[k];
+            P.rm_diag[m + k] = O.rm_diag[k] < 0 ? -1 : (int)(ent0[b] + O.rm_diag[k]);
+        }
+        std::copy(Bs[b].rows.begin(), Bs[b].rows.end(), P.vrows.begin() + row0[b]);
+        std::memcpy(P.pack.data() + (size_t)unit0[b] * kLongUnit, O.bytes.data(), O.bytes.size());
+    });
     P.chunk_row0.push_back((int64_t)P.rm_start.size());
     return HEC_OK;
 }
