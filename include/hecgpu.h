@@ -141,7 +141,11 @@ typedef struct {
                            results; for profilers that cannot see the kernels
                            of a graph with conditional nodes                */
     int64_t spin_limit; /* polls of a device wait before HEC_ERR_TIMEOUT;
-                           0 = default (about a second)                      */
+                           0 = default.  A wait also ends after two seconds,
+                           and a wait that ran out ends the solve.  Negative
+                           (krylov_solve): fault injection, the applies issue
+                           no copy and their waits run out after that many
+                           polls                                             */
 } hec_solve_opts_t;
 
 #define HEC_X0_ZERO 1
@@ -389,8 +393,8 @@ int hec_debug_record(int32_t *record, int32_t clear);
 /* z = M^{-1} r (Eq. 7 with M = the RAS combination of L_b U_b): every block
  * gathers r on V_b, solves L_b then U_b level by level, and writes z on its
  * owned rows only.  r, z: device arrays of n doubles, r != z.  Needs
- * level_schedule.  Waits are bounded by spin_limit polls (0 = default); a
- * wait that runs out is reported by hec_precond_status. */
+ * level_schedule.  Waits are bounded by spin_limit polls (0 = default)
+ * and by two seconds; a wait that runs out is reported by hec_precond_status. */
 int hec_precond_apply(hec_precond_t M, const double *r, double *z, int64_t spin_limit,
                       void *stream);
 /* Synchronise the stream and return (and clear) the device error word of

@@ -544,6 +544,7 @@ struct Solver {
     uint64_t matrix_id = 0;
     int method = 0, restart = 0;
     bool mixed = false; // GMRES with FP32 inner cycles and FP64 refinement
+    long long spin = kDefaultSpin; // waits of the preconditioner applies (< 0: nothing is issued)
     int n = 0;
     int64_t ldv = 0;
     DevBuf ws, ws32, st_buf;
@@ -638,7 +639,7 @@ int seq_precond(const hec_precond_s *M, Solver &S, const void *in, void *out, in
             return fail(HEC_ERR_INVALID, "bad typed vector op");
         return check_launch("jacobi");
     }
-    TrsvArgs a = trsv_args(M, M->lay[S.mixed ? 1 : 0], kDefaultSpin);
+    TrsvArgs a = trsv_args(M, M->lay[S.mixed ? 1 : 0], S.spin);
     a.r = in;
     a.z = out;
     a.st = S.st;
@@ -1122,21 +1123,22 @@ int solver_vecs64(int method, int restart, bool mixed)
 int solver_vecs32(int restart, bool mixed) { return mixed ? (restart + 1) + 4 : 0; }
 
 // The solver (workspace, graph) cached in the handles for these arguments.
-Solver *cached_solver(hec_matrix_s *A, hec_precond_s *M, int method, int restart, bool mixed)
+Solver *cached_solver(hec_matrix_s *A, hec_precond_s *M, int method, int restart, bool mixed,
+                      long long spin = kDefaultSpin)
 {
     auto &cache = M ? M->solvers : A->solvers;
     for (auto &p : cache)
-        if (p->matrix_id == A->id && p->method == method && p->mixed == mixed &&
+        if (p->matrix_id == A->id && p->method == method && p->mixed == mixed && p->spin == spin &&
             (method != HEC_GMRES || p->restart == restart))
             return p.get();
     return nullptr;
 }
 
 int make_solver(hec_matrix_s *A, hec_precond_s *M, int method, int restart, bool mixed,
-                cudaStream_t s, Solver *&out)
+                long long spin, cudaStream_t s, Solver *&out)
 {
     auto &cache = M ? M->solvers : A->solvers;
-    if (Solver *c = cached_solver(A, M, method, restart, mixed)) {
+    if (Solver *c = cached_solver(A, M, method, restart, mixed, spin)) {
         out = c;
         return HEC_OK;
     }
@@ -1145,6 +1147,7 @@ int make_solver(hec_matrix_s *A, hec_precond_s *M, int method, int restart, bool
     S->method = method;
     S->restart = restart;
     S->mixed = mixed;
+    S->spin = spin;
     S->n = A->hec.n;
     S->ldv = ((int64_t)S->n + 31) / 32 * 32;
     const int64_t nv = S->ldv;
@@ -2203,7 +2206,8 @@ int krylov_solve(hec_matrix_t A, hec_precond_t M, const double *b, double *x, do
                 HEC_TRY(ensure_precond_f32(M, s));
         }
         Solver *S = nullptr;
-        HEC_TRY(make_solver(A, M, o.method, restart, mixed, s, S));
+        HEC_TRY(make_solver(A, M, o.method, restart, mixed,
+                            o.spin_limit < 0 ? o.spin_limit : kDefaultSpin, s, S));
         const int n = S->n;
         const size_t vb = sizeof(double) * (size_t)n;
         // state header

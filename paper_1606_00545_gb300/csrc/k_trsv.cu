@@ -114,6 +114,34 @@ __device__ __noinline__ void debug_fail(int *err, int code, int c, int val, int 
 // in microseconds, this only guarantees that the CTA never waits forever.
 constexpr long long kDrainPolls = 1ll << 24;
 
+// A wait ran out: the handle's error word, and the end of the solve that this
+// apply is part of -- its loop would otherwise go on to its budget of steps,
+// each with the same wait.
+__device__ __forceinline__ void report_timeout(const TrsvArgs &a)
+{
+    atomicExch(a.err, HEC_ERR_TIMEOUT);
+    if (a.st) {
+        a.st->err = HEC_ERR_TIMEOUT;
+        a.st->done = 1;
+    }
+}
+
+// Polls (with a pause between them) until the progress counter of a neighbouring
+// part reaches `need`; `seen` is the value seen last.
+__device__ __forceinline__ bool progress_wait(const uint32_t *ctr, int &seen, int need,
+                                              long long limit)
+{
+    if (seen >= need || (seen = (int)ld_acquire_cluster_u32(ctr)) >= need)
+        return true;
+    const long long t0 = clock64();
+    for (long long it = 1; it < limit && clock64() - t0 < kWaitCycles; ++it) {
+        __nanosleep(32);
+        if ((seen = (int)ld_acquire_cluster_u32(ctr)) >= need)
+            return true;
+    }
+    return false;
+}
+
 // A chunk in shared memory (layout written by trsv_layout.cpp; T is the
 // value type, double or float):
 //   [0, 16)   nrows, nwarps, first position, flags (bit 0: U pass, bit 1: exports)
@@ -565,16 +593,10 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
                 // import slots its exports overwrite have been read
                 const unsigned char *ch = stages + (size_t)sh * a.stage_bytes;
                 const int2 need = *reinterpret_cast<const int2 *>(ch + (FW > 0 ? 16 : 96));
-                long long it = 0;
                 // polls back off, leaving the issue slots to the solving warps;
                 // none where the progress seen last covers the chunk
-                while (seen0 < need.x && (seen0 = (int)ld_acquire_cluster_u32(&ctr[0])) < need.x &&
-                       ++it < limit)
-                    __nanosleep(32);
-                while (seen1 < need.y && (seen1 = (int)ld_acquire_cluster_u32(&ctr[1])) < need.y &&
-                       ++it < limit)
-                    __nanosleep(32);
-                late = it >= limit;
+                late = !progress_wait(&ctr[0], seen0, need.x, limit) ||
+                       !progress_wait(&ctr[1], seen1, need.y, limit);
             }
             // (the vote also orders every lane's landed copies before the release)
             if (__any_sync(0xffffffffu, late))
@@ -662,7 +684,7 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
             const uint32_t to_prev = has_prev ? mapa_shared(smem_u32(&ctr[1]), part - 1) : 0;
             const uint32_t to_next = has_next ? mapa_shared(smem_u32(&ctr[0]), part + 1) : 0;
             uint32_t pub = 0;
-            long long it = 0;
+            long long it = 0, t0 = clock64(); // since the last change of the count
             while (pub < (uint32_t)nch) {
                 const uint32_t v = ld_acquire_cta_u32(&s_done);
                 if (v > pub) {
@@ -673,7 +695,9 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
                         st_relaxed_cluster_u32(to_next, v);
                     pub = v;
                     it = 0;
-                } else if (*reinterpret_cast<volatile int *>(&s_err) || ++it >= limit) {
+                    t0 = clock64();
+                } else if (*reinterpret_cast<volatile int *>(&s_err) || ++it >= limit ||
+                           clock64() - t0 >= kWaitCycles) {
                     failed = 1;
                     break;
                 } else {
@@ -1006,11 +1030,8 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
         for (int c = first; c < issued; ++c)
             bounded_wait(&full[c % S], (uint32_t)(c / S) & 1u, kDrainPolls);
     }
-    if (failed) {
-        atomicExch(a.err, HEC_ERR_TIMEOUT);
-        if (a.st)
-            a.st->err = HEC_ERR_TIMEOUT;
-    }
+    if (failed)
+        report_timeout(a);
     // no CTA leaves while a neighbour may still store into its shared memory
     if (clustered)
         cluster_sync_all();
@@ -1270,11 +1291,8 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
         for (int c = first; c < issued; ++c)
             bounded_wait(&full[c % S], (uint32_t)(c / S) & 1u, kDrainPolls);
     }
-    if (failed) {
-        atomicExch(a.err, HEC_ERR_TIMEOUT);
-        if (a.st)
-            a.st->err = HEC_ERR_TIMEOUT;
-    }
+    if (failed)
+        report_timeout(a);
 }
 
 // ------------------------------------------------------------------ long-row kernel
@@ -1450,11 +1468,8 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
         for (int c = first; c < issued; ++c)
             bounded_wait(&full[c % S], (uint32_t)(c / S) & 1u, kDrainPolls);
     }
-    if (failed) {
-        atomicExch(a.err, HEC_ERR_TIMEOUT);
-        if (a.st)
-            a.st->err = HEC_ERR_TIMEOUT;
-    }
+    if (failed)
+        report_timeout(a);
 }
 
 // The dynamic shared memory limit is a process-wide attribute of the kernel:

@@ -89,9 +89,19 @@ __device__ __forceinline__ uint64_t l2_evict_first_policy()
     return pol;
 }
 
+// Cycles after which a device wait gives up, whatever its limit of polls: two
+// seconds at 2.07 GHz.  A poll of an mbarrier may itself suspend the thread for
+// an unknown time, so a number of polls alone is no bound in time.
+constexpr long long kWaitCycles = 1ll << 32;
+
+// Wait for a phase: at most `limit` polls, and at most kWaitCycles.  (The first
+// poll alone is the common path: no clock is read for it.)
 __device__ __forceinline__ bool bounded_wait(uint64_t *bar, uint32_t parity, long long limit)
 {
-    for (long long it = 0; it < limit; ++it)
+    if (mbar_try_wait(bar, parity))
+        return true;
+    const long long t0 = clock64();
+    for (long long it = 1; it < limit && clock64() - t0 < kWaitCycles; ++it)
         if (mbar_try_wait(bar, parity))
             return true;
     return false;
