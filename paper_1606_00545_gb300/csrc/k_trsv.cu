@@ -1384,7 +1384,9 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
         // copies the unit of group g and forms its addresses; the stage is
         // free once every warp has its unit
         auto fetch = [&](int g) -> bool {
-            if (!bounded_wait(&full[s], par, limit)) {
+            // a vote: what follows (the unit's shuffles and barriers) is the whole
+            // warp's, and lanes that disagreed would end in different barriers
+            if (__any_sync(0xffffffffu, !bounded_wait(&full[s], par, limit))) {
                 *vfail = 1;
                 return false;
             }

@@ -55,3 +55,27 @@ def test_timeout_ends_the_solve(H, name, method, mixed, eager):
                           flags=flags)
     assert info["status"] == H.OK and info["rel_resid"] <= 1e-8
     assert H.hec_precond_status(P) == H.OK
+
+
+@pytest.mark.parametrize("name", ["long"])
+def test_waits_that_end_while_copies_land(H, name):
+    """Limits of a few polls: the waits end while the copies are landing, so
+    warps and lanes may see different outcomes.  Every apply returns, with a
+    timeout or with the full result, and the next one is right."""
+    import torch
+    A, M, P = system(H, name, 2)
+    r = synth.rhs_uniform(A.n, 1)
+    for dt, ap in ((torch.float32, H.hec_precond_apply_f32), (torch.float64, H.hec_precond_apply)):
+        rd = torch.tensor(r, dtype=dt, device="cuda:0")
+        z0 = torch.empty_like(rd)
+        ap(P, rd, z0)
+        assert H.hec_precond_status(P) == H.OK
+        z = torch.empty_like(rd)
+        for limit in [1] * 8 + [2, 3, 4, 6, 8, 12, 16, 24, 32, 64, 128, 256, 1024]:
+            ap(P, rd, z, spin_limit=limit)
+            st = H.hec_precond_status(P)
+            assert st in (H.OK, H.ERR_TIMEOUT)
+            if st == H.OK:
+                assert torch.equal(z, z0), limit
+        ap(P, rd, z)
+        assert H.hec_precond_status(P) == H.OK and torch.equal(z, z0)
