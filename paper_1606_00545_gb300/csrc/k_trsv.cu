@@ -778,6 +778,7 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
             T *own = nullptr, *gout = nullptr;
             T acc = T(0);
             bool rows = false, mine = false, exports = false;
+            bool landed = false; // the chunk copied last had been handed over
             // FP32, unsplit blocks: the set's last warp (with the shortest or
             // no rows) confirms a chunk's handover a level before the set
             // that copies it, so that the copy starts right after the barrier
@@ -803,9 +804,9 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
             auto fetch = [&](int c) {
                 const unsigned char *ch = stages + (size_t)s * a.stage_bytes;
                 if (ahead) {
-                    const int fail = *vfail;
+                    landed = !*vfail;
                     const int4 hdr = *reinterpret_cast<const int4 *>(ch);
-                    rows = !fail && w < hdr.y; // warps past the chunk's last one hold no rows
+                    rows = landed && w < hdr.y; // warps past the chunk's last one hold no rows
                     if (rows)
                         load_fixed<T, FW>(ch, hdr, rhs + (size_t)s * kThreads, w, lane, U, exps,
                                           R);
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
                 } else {
                     if (gout)
                         *gout = acc;
-                    rows = confirm(s, hpar);
+                    rows = landed = confirm(s, hpar);
                     if (rows) {
                         const int4 hdr = *reinterpret_cast<const int4 *>(ch);
                         rows = w < hdr.y;
@@ -902,9 +903,11 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
                     confirm(wrap ? 0 : s + 1, wrap ? hpar ^ 1u : hpar);
                 }
             };
-            // the stage of a chunk copied before the last barrier is free
+            // the stage of a chunk copied before the last barrier is free (not
+            // that of one whose wait ran out: its copy may be in flight, and the
+            // issuer, finding no free stage, gives up too)
             auto free_stage = [&](int c) {
-                if (row == 0 && c < c1)
+                if (row == 0 && c < c1 && landed)
                     mbar_arrive(&empty[s]);
             };
 #ifdef HEC_DEBUG
@@ -1175,11 +1178,12 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
         int nrows = 0;
         uint32_t xa[FW + 1]; // shared addresses of the dependencies and the own slot
         bool rows = false, mine = false, upper = false;
+        bool landed = false; // the chunk copied last lies in a group that landed
         // copies this set's next chunk, at (ls, lph, lk), once its group has
         // landed (after the first barrier, only the chunk that opens a group
         // asks: the other sets copy from it in later levels)
         auto fetch = [&](bool ask) {
-            rows = false;
+            rows = landed = false;
             if (*vfail) // a group that never landed: nothing is read from it
                 return;
             if (ask && !bounded_wait(&full[ls], lph, limit)) {
@@ -1197,13 +1201,15 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
                 iv[v] = (reinterpret_cast<const uint4 *>(blkp + F::idx()) + lane)[v * 32];
             dinv = reinterpret_cast<const T *>(blkp + F::dinv())[lane];
             nrows = hdr.x;
+            landed = true;
             rows = w < hdr.y; // warps past the chunk's last one idle
         };
         // chunk c's slots as shared addresses; the chunk that opens a group
         // frees the stage of the one before (its last chunk was copied at least
-        // a barrier ago)
+        // a barrier ago; after a wait that ran out nothing is freed: a copy may
+        // be in flight, and the issuer, finding no free stage, gives up too)
         auto prepare = [&](int c) {
-            if (row == 0 && lk == 0 && c > 0 && c < nch)
+            if (row == 0 && lk == 0 && c > 0 && landed)
                 mbar_arrive(&empty[ls == 0 ? S - 1 : ls - 1]);
 #pragma unroll
             for (int k = 0; k <= FW; ++k) { // vectors of 8 uint16
@@ -1260,7 +1266,7 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
             if (c + kResSets < nch)
                 fetch(lk == 0);
             else
-                rows = false;
+                rows = landed = false;
             solvers_sync<NT>();
             // ---- level c + 2
             if (c + 2 >= nch)

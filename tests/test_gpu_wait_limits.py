@@ -57,7 +57,7 @@ def test_timeout_ends_the_solve(H, name, method, mixed, eager):
     assert H.hec_precond_status(P) == H.OK
 
 
-@pytest.mark.parametrize("name", ["long"])
+@pytest.mark.parametrize("name", ["streamed", "split", "resident", "long"])
 def test_waits_that_end_while_copies_land(H, name):
     """Limits of a few polls: the waits end while the copies are landing, so
     warps and lanes may see different outcomes.  Every apply returns, with a
