@@ -302,10 +302,19 @@ __device__ __forceinline__ void solvers_set_sync(int set)
 // GB300: 19 cycles for 4 warps, the AND-reducing form 60; so the two-set loops
 // use this one.  They do not leave early on a failed wait: it sets a shared
 // word, and from then on a set loads nothing more, so the remaining levels
-// are barriers only.
-template <int NT> __device__ __forceinline__ void solvers_sync()
+// are barriers only.  bar.sync is an aligned barrier, counted by the warp: a
+// warp that reached it in two parts would be counted twice, and the set would
+// be out of step from then on, with no bound on its last barrier.  The waits
+// before it poll lane by lane, so the warp converges first (128^3 FP64 apply
+// 327.7 us without, 327.9 with).
+template <int NT> __device__ __forceinline__ void solvers_sync_converged()
 {
     asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
+}
+template <int NT> __device__ __forceinline__ void solvers_sync()
+{
+    __syncwarp();
+    solvers_sync_converged<NT>();
 }
 
 // ------------------------------------------------------------------ generic format
@@ -1186,7 +1195,9 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
             rows = landed = false;
             if (*vfail) // a group that never landed: nothing is read from it
                 return;
-            if (ask && !bounded_wait(&full[ls], lph, limit)) {
+            // a vote: the warp stays converged for the barriers (a __syncwarp at
+            // every barrier instead: 64^2 ILU(0) 49.1 us, 46.4 so)
+            if (ask && __any_sync(0xffffffffu, !bounded_wait(&full[ls], lph, limit))) {
                 *vfail = 1;
                 return;
             }
@@ -1234,13 +1245,13 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
         if (set == 0)
             prepare(c);
         // the gather above is complete too
-        solvers_sync<NT>();
+        solvers_sync_converged<NT>();
         for (int l = 0; l < c && l < nch; ++l) { // the levels before this set's first
             if (l == c - 1)
                 prepare(c);
             else if (c < nch)
                 fetch(lk == 0);
-            solvers_sync<NT>();
+            solvers_sync_converged<NT>();
         }
         while (c < nch) {
             // ---- level c
@@ -1258,7 +1269,7 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
                 if (mine)
                     sts(xa[FW], acc);
             }
-            solvers_sync<NT>();
+            solvers_sync_converged<NT>();
             // ---- level c + 1
             if (c + 1 >= nch)
                 break;
@@ -1267,15 +1278,15 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
                 fetch(lk == 0);
             else
                 rows = landed = false;
-            solvers_sync<NT>();
+            solvers_sync_converged<NT>();
             // ---- level c + 2
             if (c + 2 >= nch)
                 break;
             prepare(c + kResSets);
-            solvers_sync<NT>();
+            solvers_sync_converged<NT>();
             c += kResSets;
         }
-        solvers_sync<NT>();
+        solvers_sync_converged<NT>();
         failed = *vfail;
         if (!failed)
             for (int i0 = blk.own0 + t; i0 < blk.own1; i0 += kBatch * NT) {
@@ -1415,6 +1426,7 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
             __syncwarp();
             if (lane == 0)
                 mbar_arrive(&empty[s]);
+            __syncwarp(); // the barriers before the unit
             if (++s == S) {
                 s = 0;
                 par ^= 1u;
@@ -1423,10 +1435,13 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
         };
         int passed = 0;
         bool have = ng > 0 && fetch(0);
-        solvers_sync<NT>(); // the gather above is complete
+        // (The warp is converged at every barrier from here on: by the ends of
+        // fetch and of a unit's solve.  A __syncwarp at the barriers themselves
+        // costs 72^3 irregular 27-point 353-373 us instead of 301.)
+        solvers_sync_converged<NT>(); // the gather above is complete
         for (int g = 0; g < ng && have; ++g) {
             for (int nb = (flags >> 7) & 63; nb > 0; --nb, ++passed)
-                solvers_sync<NT>();
+                solvers_sync_converged<NT>();
             float y[kLongPerLane], acc, x;
 #pragma unroll
             for (int k = 0; k < kLongPerLane; ++k)
@@ -1444,8 +1459,9 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
             }
             if (flags & 64)
                 sts(xa[kLongPerLane], acc * mul);
+            __syncwarp();
             if (flags >> 13 & 1) { // the level goes on without this warp
-                solvers_sync<NT>();
+                solvers_sync_converged<NT>();
                 ++passed;
             }
             if (g + 1 < ng)
@@ -1453,8 +1469,8 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
         }
         // every warp passes every level's barrier, also after a failed wait
         for (; passed < nlev; ++passed)
-            solvers_sync<NT>();
-        solvers_sync<NT>();
+            solvers_sync_converged<NT>();
+        solvers_sync_converged<NT>();
         failed = *vfail;
         if (!failed)
             for (int i0 = blk.own0 + t; i0 < blk.own1; i0 += kBatch * NT) {
