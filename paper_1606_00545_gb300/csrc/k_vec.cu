@@ -320,13 +320,18 @@ __device__ __forceinline__ double warp_sum_group(double (&v)[kGroup], int lane)
     return t;
 }
 
-// h[i] = (V_i, w), i < k.  Grid (row blocks, vector groups); every CTA keeps
-// kGroup running sums per thread (in T) and reduces them once at the end (in
-// FP64, fixed order).  In FP64 the multiply-adds bound it: k n of them at two
-// per cycle and SM (2,097,152 x 30: 101 us at 2.07 GHz, the HBM stream 78),
-// so the grid holds only as many CTAs as run at once and each pays one
-// reduction for many rows, and two rows' loads are in flight per thread:
-// 166 -> 121 us (k = 8: 74 -> 43).
+// h[i] = (V_i, w), i < k.  A CTA takes one row block of one group of kGroup
+// vectors, keeps kGroup running sums per thread (in T) and reduces them once at
+// the end (in FP64, fixed order).  In FP64 the multiply-adds bound it: k n of
+// them at two per cycle and SM (2,097,152 x 30: 101 us at 2.07 GHz, the HBM
+// stream 78), so the grid holds only as many CTAs as run at once and each pays
+// one reduction for many rows, and two rows' loads are in flight per thread:
+// 166 -> 121 us (k = 8: 74 -> 43).  Inside a GMRES step the launch is sized
+// for a whole cycle and k is the step's: the CTAs are split over the groups
+// that k has, so that the first steps of a cycle use every SM as well (by the
+// cycle's groups, restart 128 left 17 CTAs reading the first eight vectors:
+// 128^3, 8 steps of GMRES(128) 6.4 ms, 1.9 so; 30 steps of GMRES(30) 12.9 and
+// 11.0).
 template <class T> __global__ void __launch_bounds__(kThreads) k_multidot(BasisArgs a)
 {
     count_launch(a.st);
@@ -340,17 +345,21 @@ template <class T> __global__ void __launch_bounds__(kThreads) k_multidot(BasisA
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     __shared__ double sh[kThreads / 32][kGroup];
     __shared__ int s_last;
-    const int g0 = blockIdx.y * kGroup;
+    // row blocks per group: as many as there are rows or CTAs for
+    const int rb = a.row_ctas ? a.row_ctas
+                              : min((a.n - 1) / kThreads + 1,
+                                    (int)gridDim.x / ((k + kGroup - 1) / kGroup));
+    const int g0 = (int)blockIdx.x / rb * kGroup, rblk = (int)blockIdx.x % rb;
     if (g0 < k) {
         T acc[kGroup];
 #pragma unroll
         for (int q = 0; q < kGroup; ++q)
             acc[q] = T(0);
         const uint64_t pol = basis_policy();
-        const int stride = gridDim.x * kThreads;
+        const int stride = rb * kThreads;
         const T *Vg = V + (int64_t)g0 * a.ldv;
         const int cnt = min(kGroup, k - g0); // vectors of this group
-        int i = blockIdx.x * kThreads + threadIdx.x;
+        int i = rblk * kThreads + threadIdx.x;
         for (; i < a.n - stride; i += 2 * stride) { // two rows' loads in flight
             T v0[kGroup], v1[kGroup];
 #pragma unroll
@@ -389,13 +398,13 @@ template <class T> __global__ void __launch_bounds__(kThreads) k_multidot(BasisA
         // partials layout: [vector][row block]
         const int q = g0 + threadIdx.x;
         if (q < k)
-            a.red.partials[(size_t)q * gridDim.x + blockIdx.x] = t;
+            a.red.partials[(size_t)q * rb + rblk] = t;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         unsigned tk = atomicAdd(a.red.ticket, 1u);
-        s_last = (tk == gridDim.x * gridDim.y - 1);
+        s_last = (tk == gridDim.x - 1);
     }
     __syncthreads();
     if (!s_last)
@@ -406,9 +415,9 @@ template <class T> __global__ void __launch_bounds__(kThreads) k_multidot(BasisA
         const int q = q0 + threadIdx.x / 8, part = threadIdx.x % 8;
         double t = 0.0;
         if (q < k) {
-            const double *pq = &a.red.partials[(size_t)q * gridDim.x];
+            const double *pq = &a.red.partials[(size_t)q * rb];
 #pragma unroll 4
-            for (unsigned c = part; c < gridDim.x; c += 8)
+            for (int c = part; c < rb; c += 8)
                 t += __ldcg(&pq[c]);
         }
 #pragma unroll
@@ -427,20 +436,22 @@ template <class T> __global__ void __launch_bounds__(kThreads) k_multidot(BasisA
         *a.red.ticket = 0u;
 }
 
-int launch_multidot(const BasisArgs &a, int sms, cudaStream_t s, bool fp32)
+int launch_multidot(BasisArgs a, int sms, cudaStream_t s, bool fp32)
 {
     // a.k is the number of vectors, or an upper bound of it when k_from_st.
     // Row blocks: FP64, at most kMultidotCtas CTAs per SM over all groups;
     // FP32, two per SM and group -- more rows per thread would lengthen its
     // FP32 running sums.
     const int groups = (a.k + kGroup - 1) / kGroup;
-    const int cap = fp32 ? 2 * sms : max(1, sms * kMultidotCtas / groups);
     const int need = (int)(((int64_t)a.n + kThreads - 1) / kThreads);
-    dim3 g(min(need, cap), groups);
-    if (fp32)
-        k_multidot<float><<<g, kThreads, 0, s>>>(a);
-    else
-        k_multidot<double><<<g, kThreads, 0, s>>>(a);
+    if (fp32) {
+        a.row_ctas = min(need, 2 * sms);
+        k_multidot<float><<<a.row_ctas * groups, kThreads, 0, s>>>(a);
+        return 0;
+    }
+    a.row_ctas = 0; // split on the device
+    const int64_t most = max(sms * kMultidotCtas, groups);
+    k_multidot<double><<<(int)min((int64_t)need * groups, most), kThreads, 0, s>>>(a);
     return 0;
 }
 

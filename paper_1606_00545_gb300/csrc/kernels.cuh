@@ -154,12 +154,13 @@ struct BasisArgs {
     double *result;
     int op;
     SolverState *st;
+    int row_ctas;          // projections: CTAs per vector group (0: split on the device)
 };
 // CTAs per SM of an FP64 projection, over all vector groups: each CTA reads
 // long runs and pays its reduction once.  n = 2,097,152, k = 30: 121 us with 2,
 // 123 with 3, 151 with 4.
 constexpr int kMultidotCtas = 2;
-int launch_multidot(const BasisArgs &a, int sms, cudaStream_t s, bool fp32 = false);
+int launch_multidot(BasisArgs a, int sms, cudaStream_t s, bool fp32 = false);
 // wout = w - sum_i coef[i] V_i  (with_norm: + fused (wout, wout) -> op)
 int launch_basis_update(const BasisArgs &a, bool with_norm, int grid, cudaStream_t s,
                         bool fp32 = false);
