@@ -27,6 +27,7 @@ import os
 import statistics
 import subprocess
 import sys
+import threading
 import time
 
 import numpy as np
@@ -652,7 +653,9 @@ def c5_section(H, n_lambda=C5_REQUESTS, n_quarter_lambda=C5_REQUESTS, n_half=40,
         got = []
         while len(got) < len(pool):
             got += S.poll(wait_ms=100)
-        assert all(r["status"] == H.OK for r in got), got
+        # a system near GMRES(30) stagnation may spend its budget of steps: it is
+        # resident all the same (the first streams' status_counts show such solves)
+        assert all(r["status"] in (H.OK, H.MAXIT) for r in got), got
         return time.perf_counter() - t
 
     def open_loop(S, rate, req, keyed):
@@ -759,6 +762,46 @@ def c5_section(H, n_lambda=C5_REQUESTS, n_quarter_lambda=C5_REQUESTS, n_half=40,
 
 
 # ------------------------------------------------------------------ our arm
+# The sections after the headline take about 90 s; by this limit the line is
+# printed with those that are done.
+SECTIONS_LIMIT_S = 600.0
+
+
+def run_sections(line, sections, limit_s, emit, leave):
+    """Runs the (key, function) sections into ``line`` and emits it, once: at
+    the end, or after ``limit_s`` seconds without the sections that are not
+    done, named under "unfinished" (then ``leave`` ends the process).  A
+    section that raises leaves its error in its place."""
+    lock = threading.Lock()
+    emitted = []
+
+    def finish(late):
+        with lock:
+            if emitted:
+                return
+            emitted.append(True)
+            if late:
+                line["unfinished"] = [n for n, _ in sections if n not in done]
+            emit(line)
+            if late:
+                leave()
+
+    done = set()
+    timer = threading.Timer(limit_s, finish, (True,))
+    timer.daemon = True
+    timer.start()
+    for name, fn in sections:
+        try:
+            res = fn()
+        except Exception as e:  # the other measurements are kept
+            res = {"error": ("%s: %s" % (type(e).__name__, e))[:500]}
+        with lock:
+            line[name] = res
+            done.add(name)
+    timer.cancel()
+    finish(False)
+
+
 def run_ours(args, rank, world, local_rank):
     import torch
     from paper_1606_00545_gb300 import build
@@ -905,17 +948,8 @@ def run_ours(args, rank, world, local_rank):
     H.hec_refactor(Ah, P, v1)  # back to the benchmark's matrix
     pinf = P.info()
     trsv_bytes32 = trsv_method_bytes(H, P, 4)
-    skip = set(filter(None, args.skip.split(",")))
-    c1 = (c1_section(H, torch, dev, rank == 0 and not args.no_cpu_baseline)
-          if "c1" not in skip else None)
-    c3 = c3_section(H, torch, dev, timed) if "c3" not in skip else None
-    c4 = c4_section(H, torch, dev, timed, peak) if "c4" not in skip else None
-    c5 = c5_section(H) if "c5" not in skip else None
-
-    if rank != 0:
-        return
     cpu = None
-    if not args.no_cpu_baseline:
+    if rank == 0 and not args.no_cpu_baseline:
         rate, it, dt, cpu_setup, cpu_apply = cpu_sample(A, b, CPU_SAMPLE_ITERS)
         cpu = {"value": rate, "unit": "iter/s", "cores": 1, "kind": "oracle",
                "sample": "%d BiCGSTAB iterations of the full 128^3 workload from x0 = 0 "
@@ -969,13 +1003,22 @@ def run_ours(args, rank, world, local_rank):
                          "trsv_needed_rows_bytes": pinf["apply_bytes_f32"],
                          "spmv_ms": ms_s32 / reps,
                          "spmv_gbs": (A.nnz * 8 + A.n * 8) / (ms_s32 * 1e-3 / reps) / 1e9},
-        "c1_latency": c1,
-        "c3_irregular_mixed": c3,
-        "c4_batched": c4,
-        "c5_serving": c5,
+        "c1_latency": None,
+        "c3_irregular_mixed": None,
+        "c4_batched": None,
+        "c5_serving": None,
         "cpu_baseline": cpu,
     }
-    print(json.dumps(line), flush=True)
+    skip = set(filter(None, args.skip.split(",")))
+    sections = [
+        ("c1_latency", lambda: c1_section(H, torch, dev, rank == 0 and not args.no_cpu_baseline)),
+        ("c3_irregular_mixed", lambda: c3_section(H, torch, dev, timed)),
+        ("c4_batched", lambda: c4_section(H, torch, dev, timed, peak)),
+        ("c5_serving", lambda: c5_section(H)),
+    ]
+    run_sections(line, [(n, f) for n, f in sections if n[:2] not in skip], SECTIONS_LIMIT_S,
+                 lambda l: print(json.dumps(l), flush=True) if rank == 0 else None,
+                 lambda: os._exit(0))
 
 
 # ------------------------------------------------------------------ Table 4 / 5 sweep

@@ -110,3 +110,32 @@ def test_c4_bytes_charges_the_third_gram_schmidt_pass():
     want = sum(30 * (29 / 2 + 3) * float(Bs.sys_ptr[s + 1] - Bs.sys_ptr[s]) * 4 * 4
                for s in range(3))
     assert abs(extra - want) <= 1e-9 * want
+
+
+def test_sections_failing_or_late_do_not_lose_the_line():
+    """The line is emitted once, with every section that is done: a section
+    that raises leaves its error, one that outlasts the limit is named."""
+    import threading
+
+    out, left = [], []
+    line = {"value": 1.0, "a": None, "b": None}
+
+    def broken():
+        raise AssertionError("no solve converged")
+
+    bench.run_sections(line, [("a", lambda: 5), ("b", broken)], 60.0,
+                       lambda l: out.append(dict(l)), lambda: left.append(1))
+    assert out == [{"value": 1.0, "a": 5, "b": {"error": "AssertionError: no solve converged"}}]
+    assert not left
+    # a late section: the limit's thread emits the line and leaves
+    out.clear()
+    gate = threading.Event()
+    line = {"value": 1.0, "a": None, "b": None}
+
+    def leave():
+        left.append(1)
+        gate.set()  # (a real caller ends the process here)
+
+    bench.run_sections(line, [("a", lambda: 5), ("b", lambda: gate.wait(30))], 0.2,
+                       lambda l: out.append(dict(l)), leave)
+    assert out == [{"value": 1.0, "a": 5, "b": None, "unfinished": ["b"]}] and left == [1]
