@@ -428,15 +428,17 @@ int pack_layout(const hec_precond_s *M, int idx, TrsvPack &P, int &fixed_width, 
             }
         }
         // Rows too long for the fixed-slot formats, FP32: the long-row kernel
-        // where the block's vector fits beside three stages and the streamed
-        // kernel would not split a block.  LRULE
+        // where the block's vector fits beside its stages and the streamed
+        // kernel would not split a block.
         if (M->trsv_kernel == HEC_TRSV_AUTO && idx == 1 && trsv_uniform_width(longest) == 0 &&
             maxnv < kLongSlots && layout_parts(M, idx) == 1) {
             const int stage = kLongWarps * kLongUnit;
             nstages = M->host_only
-                          ? (trsv_res_smem_bytes(stage, 3, maxnv + 1, vb) <= 226 * 1024 ? 3 : 0)
+                          ? (trsv_res_smem_bytes(stage, kLongStages, maxnv + 1, vb) <= 226 * 1024
+                                 ? kLongStages
+                                 : 0)
                           : trsv_res_stages_for(stage, maxnv + 1, vb);
-            if (nstages > 0) {
+            if (nstages >= kLongStages) {
                 fixed_width = 0;
                 return pack_trsv_long(M->blocks, P, msg);
             }

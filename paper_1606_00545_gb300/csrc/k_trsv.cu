@@ -1322,11 +1322,18 @@ __global__ void __launch_bounds__(kResSolvers<NW> + 32, 1) k_trsv_res(TrsvArgs a
 // further back than any ring, so the streamed kernel also read them from
 // global memory: 72^3, ILU(0), 64 blocks 1,806 -> 295 us.
 // A warp's work in a level is a unit (kernels.cuh); kLongWarps units, one per
-// warp, travel in one bulk copy.  A warp holds its next unit in registers with
-// its addresses formed, passes the level barriers that come before it, solves
-// it, passes its own level's barrier and then loads the next one -- a level of
-// three units leaves each warp several levels for that.
+// warp, travel in one bulk copy.  A warp copies its next unit into registers,
+// forms its addresses and waits until the units of the earlier levels are
+// solved: every warp publishes how many units it has solved, and the lanes read
+// all warps' counts.  So a warp without a unit in a level takes no part in it,
+// and every wait between warps has its limit.
+// (A barrier of all warps per level as bar.sync, 305 us on the case above, is
+// not sound here: on a served stream of eight lanes a solve's steps changed from
+// run to run and some applies never ended, three of five runs, while the same
+// kernel with counted waits gave the same steps in every run.  As an mbarrier of
+// all warps: 553 us.  This form: 350; with 16 warps 3% more.)
 constexpr int kLongThreads = 32 * kLongWarps;
+constexpr int kLongPolls = 64; // polls between two readings of the clock
 __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
 {
     constexpr int NT = kLongThreads;
@@ -1345,12 +1352,15 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
     uint64_t *full = reinterpret_cast<uint64_t *>(
         reinterpret_cast<unsigned char *>(xs) + (((size_t)a.res_slots * sizeof(float) + 7) & ~(size_t)7));
     uint64_t *empty = full + S;
-    const int ng = blk.ngroups, nlev = blk.ring_L;
+    const int ng = blk.ngroups;
     const int *vrows = a.vrows + blk.yoff;
     const bool stall_test = a.spin_limit < 0; // fault injection: nothing is issued
     const long long limit = stall_test ? -a.spin_limit : a.spin_limit;
     const int t = threadIdx.x;
     __shared__ int s_issued, s_fail;
+    __shared__ uint32_t s_solved[kLongWarps]; // per warp: 1 + its solved units (0: not gathered yet)
+    if (t < kLongWarps)
+        s_solved[t] = 0;
     if (t == 0) {
         for (int s = 0; s < S; ++s) {
             mbar_init(&full[s], 1);
@@ -1401,8 +1411,7 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
         // copies the unit of group g and forms its addresses; the stage is
         // free once every warp has its unit
         auto fetch = [&](int g) -> bool {
-            // a vote: what follows (the unit's shuffles and barriers) is the whole
-            // warp's, and lanes that disagreed would end in different barriers
+            // a vote: what follows (the unit's waits and shuffles) is the whole warp's
             if (__any_sync(0xffffffffu, !bounded_wait(&full[s], par, limit))) {
                 *vfail = 1;
                 return false;
@@ -1426,22 +1435,53 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
             __syncwarp();
             if (lane == 0)
                 mbar_arrive(&empty[s]);
-            __syncwarp(); // the barriers before the unit
             if (++s == S) {
                 s = 0;
                 par ^= 1u;
             }
             return true;
         };
-        int passed = 0;
-        bool have = ng > 0 && fetch(0);
-        // (The warp is converged at every barrier from here on: by the ends of
-        // fetch and of a unit's solve.  A __syncwarp at the barriers themselves
-        // costs 72^3 irregular 27-point 353-373 us instead of 301.)
-        solvers_sync_converged<NT>(); // the gather above is complete
+        // this warp's count, after its stores
+        auto publish = [&](uint32_t solved) {
+            __syncwarp();
+            if (lane == 0)
+                st_release_cta_u32(&s_solved[w], 1u + solved);
+        };
+        // waits until the units below index `first` are solved (and every warp
+        // has gathered): lane l reads warp l mod kLongWarps's count
+        auto wait_for = [&](int first) -> bool {
+            const uint32_t need = 1u + (uint32_t)(first + kLongWarps - 1 - lane % kLongWarps) / kLongWarps;
+            const uint32_t *p = &s_solved[lane % kLongWarps];
+            bool ok = __all_sync(0xffffffffu, ld_relaxed_cta_u32(p) >= need);
+            long long t0 = 0;
+            for (long long left = limit - 1; !ok && left > 0; left -= kLongPolls) {
+#pragma unroll 1
+                for (int k = 0; k < kLongPolls; ++k)
+                    if ((ok = __all_sync(0xffffffffu, ld_relaxed_cta_u32(p) >= need)))
+                        break;
+                if (ok)
+                    break;
+                const long long now = clock64(); // (read once in kLongPolls polls)
+                if (t0 == 0)
+                    t0 = now;
+                if (__any_sync(0xffffffffu, now - t0 >= kWaitCycles))
+                    break;
+            }
+            fence_acq_rel_cta();
+            __syncwarp(); // every lane's reads come after every count
+            if (!ok)
+                *vfail = 1;
+            return ok;
+        };
+        publish(0);
+        bool have = true;
         for (int g = 0; g < ng && have; ++g) {
-            for (int nb = (flags >> 7) & 63; nb > 0; --nb, ++passed)
-                solvers_sync_converged<NT>();
+            have = fetch(g);
+            if (!have)
+                break;
+            have = wait_for(g * kLongWarps + w - (flags >> 7));
+            if (!have)
+                break;
             float y[kLongPerLane], acc, x;
 #pragma unroll
             for (int k = 0; k < kLongPerLane; ++k)
@@ -1459,19 +1499,10 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
             }
             if (flags & 64)
                 sts(xa[kLongPerLane], acc * mul);
-            __syncwarp();
-            if (flags >> 13 & 1) { // the level goes on without this warp
-                solvers_sync_converged<NT>();
-                ++passed;
-            }
-            if (g + 1 < ng)
-                have = fetch(g + 1);
+            publish((uint32_t)g + 1u);
         }
-        // every warp passes every level's barrier, also after a failed wait
-        for (; passed < nlev; ++passed)
-            solvers_sync_converged<NT>();
-        solvers_sync_converged<NT>();
-        failed = *vfail;
+        // the block is solved
+        failed = !have || !wait_for(ng * kLongWarps) || *vfail;
         if (!failed)
             for (int i0 = blk.own0 + t; i0 < blk.own1; i0 += kBatch * NT) {
                 int g[kBatch];

@@ -240,12 +240,13 @@ int launch_trsv(const TrsvArgs &a, cudaStream_t s, bool fp32 = false);
 // or above c / 4), aligned to G; entry j + k G is value k of its lane j.
 // Flags: bits 0-2 log2 G, bits 3-5 the largest log2 G of the unit, bit 6 the
 // row's first lane (it holds the right-hand side and stores the result), bits
-// 7-12 the level barriers the warp passes before this unit, bit 13: one more
-// right after it (its next unit lies in a later level), before that unit is
-// loaded.
-constexpr int kLongWarps = 16;      // solving warps: unit u of a block is warp u mod 16's
+// 7-15: the unit comes this many units after its level's first one (at most
+// kLongBack: then it also waits for units of its own level).
+constexpr int kLongWarps = 8;       // solving warps: unit u of a block is warp u mod 8's
 constexpr int kLongUnit = 1024;     // bytes of a unit
 constexpr int kLongPerLane = 4;     // entries per lane
+constexpr int kLongBack = 511;
+constexpr int kLongStages = 6;      // fewest stages of kLongWarps units worth running with
 constexpr int kLongSlots = 65535;   // a block has fewer rows than this
 // The first violation a debug build (HEC_DEBUG) recorded: code, program,
 // chunk, thread, value, bound, 0, 0 (all 0: none); clear resets it.

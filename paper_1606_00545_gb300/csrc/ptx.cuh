@@ -215,6 +215,18 @@ __device__ __forceinline__ uint32_t ld_acquire_cta_u32(const void *p)
     return v;
 }
 
+// A relaxed load of a shared word, for polls that a fence follows.
+__device__ __forceinline__ uint32_t ld_relaxed_cta_u32(const void *p)
+{
+    uint32_t v;
+    asm volatile("ld.relaxed.cta.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+__device__ __forceinline__ void fence_acq_rel_cta()
+{
+    asm volatile("fence.acq_rel.cta;" ::: "memory");
+}
+
 __device__ __forceinline__ void st_release_cta_u64(void *p, uint64_t v)
 {
     asm volatile("st.release.cta.shared::cta.u64 [%0], %1;" ::"r"(smem_u32(p)), "l"(v) : "memory");

@@ -846,7 +846,7 @@ void emit_resident(const BlockFactor &B, int FW, int vb, int NW, ResOut &O)
 // is already in place).
 struct LongOut {
     std::vector<unsigned char> bytes;
-    int units = 0, levels = 0, nL = 0, nU = 0, own0 = 0, own1 = 0;
+    int units = 0, nL = 0, nU = 0, own0 = 0, own1 = 0;
     std::vector<int> rm_start, rm_len, rm_diag; // per lane
     int64_t alg = 0;
 };
@@ -877,26 +877,14 @@ void emit_long(const BlockFactor &B, LongOut &O)
     O.rm_start.reserve(guess * kWarpRows);
     O.rm_len.reserve(guess * kWarpRows);
     O.rm_diag.reserve(guess * kWarpRows);
-    // per warp: the level barriers it has passed, its last unit's level and place
-    std::vector<int> passed(kLongWarps, 0), last_level(kLongWarps, -1);
-    std::vector<size_t> last_off(kLongWarps, 0);
-    // the barrier of the warp's last unit's level, before a unit of level `l`
-    auto close_last = [&](int w, int l) {
-        if (last_level[w] < 0 || last_level[w] >= l)
-            return;
-        unsigned char *rec = O.bytes.data() + last_off[w] + 512;
-        for (int q = 0; q < kWarpRows; ++q)
-            reinterpret_cast<uint16_t *>(rec + 16 * q)[5] |= 1u << 13;
-        passed[w] = last_level[w] + 1;
-        last_level[w] = -1;
-    };
     std::vector<Piece> ps;
     auto emit_level = [&]() {
         if (ps.empty())
             return;
         size_t i = 0;
+        const int first = O.units; // the level's first unit
         while (i < ps.size()) { // one unit
-            const int u = O.units++;
+            const int back = std::min(O.units++ - first, kLongBack);
             const size_t off = O.bytes.size();
             O.bytes.resize(off + kLongUnit, 0);
             const size_t m0 = O.rm_start.size();
@@ -944,18 +932,10 @@ void emit_long(const BlockFactor &B, LongOut &O)
                 }
                 ++i;
             }
-            const int w = u % kLongWarps;
-            close_last(w, O.levels);
-            const int nbar = O.levels - passed[w];
-            passed[w] = O.levels;
-            last_level[w] = O.levels;
-            last_off[w] = off;
-            rec = O.bytes.data() + off + 512;
             for (int l = 0; l < kWarpRows; ++l)
                 reinterpret_cast<uint16_t *>(rec + 16 * l)[5] =
-                    (uint16_t)(flags[l] | (maxlg << 3) | (nbar << 7));
+                    (uint16_t)(flags[l] | (maxlg << 3) | (back << 7));
         }
-        ++O.levels;
         ps.clear();
     };
     for (int pass = 0; pass < 2; ++pass) {
@@ -993,11 +973,8 @@ void emit_long(const BlockFactor &B, LongOut &O)
             start = end;
         }
     }
-    for (int w = 0; w < kLongWarps; ++w)
-        close_last(w, O.levels);
     // whole groups of kLongWarps units: the last ones idle
     while (O.units % kLongWarps != 0) {
-        const int w = O.units % kLongWarps;
         const size_t off = O.bytes.size();
         O.bytes.resize(off + kLongUnit, 0);
         O.rm_start.resize(O.rm_start.size() + kWarpRows, 0);
@@ -1008,10 +985,8 @@ void emit_long(const BlockFactor &B, LongOut &O)
             uint16_t *s = reinterpret_cast<uint16_t *>(rec + 16 * l);
             for (int k = 0; k < kLongPerLane + 1; ++k)
                 s[k] = (uint16_t)nv;
-            s[5] = (uint16_t)((O.levels - passed[w]) << 7);
             reinterpret_cast<float *>(rec + 16 * l)[3] = 1.0f;
         }
-        passed[w] = O.levels;
         ++O.units;
     }
 }
@@ -1146,8 +1121,7 @@ int pack_trsv_long(const std::vector<BlockFactor> &Bs, TrsvPack &P, std::string 
         T.chunk_end = (int)unit0[b + 1];
         T.zoff = unit0[b] / kLongWarps;
         T.ngroups = O.units / kLongWarps;
-        T.ring_L = O.levels; // level barriers of the block
-        T.ring_U = 1;
+        T.ring_L = T.ring_U = 1;
         T.yoff = row0[b];
         T.nv = Bs[b].F.n;
         T.own0 = O.own0;
