@@ -22,7 +22,7 @@
 //   - an issuer warp streams chunks into a ring of shared-memory stages with
 //     cp.async.bulk (the TMA bulk-copy engine, evict-first in L2) completing
 //     on mbarriers, S chunks ahead of the solving warps;
-//   - two gatherer warps, taking chunks in turn, gather each landed chunk's
+//   - three gatherer warps, taking chunks in turn, gather each landed chunk's
 //     right-hand sides (L pass: from r; U pass: from the L results, once the
 //     L pass is complete) with 4- or 8-byte cp.async, ahead of the solving
 //     warps, and hand the chunk over (an mbarrier per stage) once the copies
@@ -60,14 +60,18 @@ size_t trsv_smem_bytes(int stage_bytes, int nstages, int ring_slots, int vbytes)
 }
 
 // Gatherer warps of a CTA: they take the chunks in turn and keep up to
-// kGatherDepth chunks' right-hand-side gathers in flight each.  (Two, three
-// or four gatherers, depths 2 and 4: within 4% on the 128^3 case.)
-constexpr int kGatherers = 2;
+// kGatherDepth chunks' right-hand-side gathers in flight each.  Two, three and
+// four of them, FP64 / FP32 apply in us: 128^3 ILU(1) 325 / 290, 318 / 231,
+// 320 / 234; 96^3 ILU(0) 171 / 178, 151 / 150, 153 / 150; 40^3 ILU(0) in 4
+// blocks 84 / 96, 72 / 82, 72 / 82.
+constexpr int kGatherers = 3;
 constexpr int kGatherDepth = 2;
 
 constexpr int kMaxStages = 16; // of the streamed kernel
-// Shared memory and (with two gatherer warps, 640 threads) registers left on
-// the SM for the vector and reduction kernels of other streams.
+// Shared memory that the stages leave: with all but 1 KB in stages, copies run
+// further ahead than the solving warps need and the FP64 applies are slower
+// (101^3 ILU(1) 461 us, 437 so; 82^3 ILU(0) 257 and 237; FP32 within 2% but for
+// 101^3, 229 and 213).
 constexpr int kLeaveFree = 24 * 1024;
 
 int trsv_stages_for(int stage_bytes, int ring_slots, int vbytes)
@@ -458,11 +462,11 @@ __device__ __forceinline__ bool issue_chunks(const uint2 *chunks, int nch, int S
 }
 
 // Warp-specialised CTA: 8 warps (fixed-slot chunks: two sets of 8) solve rows,
-// one row per thread per chunk; the last four warps feed them.  Per chunk c
+// one row per thread per chunk; the last five warps feed them.  Per chunk c
 // in stage s = c mod S:
 //   issuer: wait empty[s] (chunk c - S released) -> arm full[s] with
 //             the chunk's byte count -> cp.async.bulk the chunk;
-//   gatherers (two warps, chunks in turn): wait full[s] -> gather
+//   gatherers (three warps, chunks in turn): wait full[s] -> gather
 //             the chunk's right-hand sides into slot s with cp.async, one
 //             commit group per chunk (a U chunk waits for ldone first: its
 //             right-hand side is the L pass's output) -> once the group has
@@ -581,9 +585,9 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
         const int gw = (t - NT - 32) / 32;
         const int lane = t % 32;
         bool ldone_seen = false;
-        // with 3 or 4 stages two of them work: the phase tests below tell a
-        // stage's uses apart when a chunk that this warp saw land was issued
-        // after the stage's last use but one was released (S >= NG)
+        // with 3 stages two of them work: the phase tests below tell a stage's
+        // uses apart when a chunk that this warp saw land was issued after the
+        // stage's last use but one was released (S >= NG; one more to spare)
         const int NG = S > kGatherers ? kGatherers : 2;
         int sg = gw; // gw < NG <= S: chunk gw lies in stage gw, phase 0
         uint32_t par = 0;
