@@ -12,8 +12,7 @@
 // for the j of row p's U part that row i holds -- with separately rounded
 // multiply and subtract (no contraction, as the host code is compiled), so
 // the factors are bit-identical to a host factorisation of the new matrix.
-#include <mutex>
-
+#include "per_device.h"
 #include "ptx.cuh"
 #include "reduce.cuh"
 
@@ -435,12 +434,13 @@ template <int LEN, bool PLAN>
 static int launch_rows(const RefactorArgs &a, int nblocks, int C, cudaStream_t s)
 {
     constexpr int smem = LEN * kThreads * (int)(sizeof(double) + sizeof(int));
-    static std::once_flag once;
-    static cudaError_t e = cudaSuccess;
-    std::call_once(once, []() {
-        e = cudaFuncSetAttribute(k_iluk_rows<LEN, PLAN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    });
-    if (e != cudaSuccess)
+    static PerDevice<cudaError_t> once;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (once.get(dev, []() {
+            return cudaFuncSetAttribute(k_iluk_rows<LEN, PLAN>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        }) != cudaSuccess)
         return -1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(nblocks * C));

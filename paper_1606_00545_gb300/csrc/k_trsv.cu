@@ -41,9 +41,9 @@
 // grid-wide synchronisation.  Every wait is bounded: a wait that runs out
 // sets the device error word, one thread waits (bounded) for the copies still
 // in flight, and the CTA returns.
-#include <mutex>
 #include <type_traits>
 
+#include "per_device.h"
 #include "ptx.cuh"
 #include "reduce.cuh"
 
@@ -1531,43 +1531,33 @@ __global__ void __launch_bounds__(kLongThreads + 32, 1) k_trsv_long(TrsvArgs a)
         report_timeout(a);
 }
 
-// The dynamic shared memory limit is a process-wide attribute of the kernel:
-// raised once to the device's opt-in maximum, so that launches of different
-// sizes from several host threads never race on it.
-template <class T, int FW, bool RES, int NW = 8> static cudaError_t prepare_trsv()
+// The dynamic shared memory limit is an attribute of the kernel on a device:
+// raised once to the device's opt-in maximum, which covers static and dynamic
+// shared memory, so that launches of different sizes from several host threads
+// never race on it.
+template <class K> static cudaError_t prepare_trsv(PerDevice<cudaError_t> &once, K kernel)
 {
-    static std::once_flag once;
-    static cudaError_t e = cudaSuccess;
-    std::call_once(once, []() {
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return once.get(dev, [&]() {
+        int optin = 0;
         cudaFuncAttributes fa{};
-        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        if (e == cudaSuccess) {
-            if constexpr (RES)
-                e = cudaFuncGetAttributes(&fa, k_trsv_res<T, FW, NW>);
-            else
-                e = cudaFuncGetAttributes(&fa, k_trsv_ras<T, FW>);
-        }
-        if (e == cudaSuccess) { // the opt-in limit covers static and dynamic shared memory
-            if constexpr (RES)
-                e = cudaFuncSetAttribute(k_trsv_res<T, FW, NW>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         optin - (int)fa.sharedSizeBytes);
-            else
-                e = cudaFuncSetAttribute(k_trsv_ras<T, FW>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         optin - (int)fa.sharedSizeBytes);
-        }
+        cudaError_t e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess)
+            e = cudaFuncGetAttributes(&fa, kernel);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     optin - (int)fa.sharedSizeBytes);
+        return e;
     });
-    return e;
 }
 
 template <class T, int FW> static int launch_t(const TrsvArgs &a, cudaStream_t s)
 {
     const size_t smem =
         trsv_smem_bytes(a.stage_bytes, a.nstages, a.ring_mask + 1 + a.import_slots, sizeof(T));
-    if (prepare_trsv<T, FW, false>() != cudaSuccess)
+    static PerDevice<cudaError_t> once;
+    if (prepare_trsv(once, k_trsv_ras<T, FW>) != cudaSuccess)
         return -1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)a.nblocks);
@@ -1587,7 +1577,8 @@ template <class T, int FW> static int launch_t(const TrsvArgs &a, cudaStream_t s
 template <class T, int FW, int NW> static int launch_res(const TrsvArgs &a, cudaStream_t s)
 {
     const size_t smem = trsv_res_smem_bytes(a.stage_bytes, a.nstages, a.res_slots, sizeof(T));
-    if (prepare_trsv<T, FW, true, NW>() != cudaSuccess)
+    static PerDevice<cudaError_t> once;
+    if (prepare_trsv(once, k_trsv_res<T, FW, NW>) != cudaSuccess)
         return -1;
     k_trsv_res<T, FW, NW><<<a.nblocks, kResSolvers<NW> + 32, smem, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -1595,20 +1586,8 @@ template <class T, int FW, int NW> static int launch_res(const TrsvArgs &a, cuda
 
 static int launch_long(const TrsvArgs &a, cudaStream_t s)
 {
-    static std::once_flag once;
-    static cudaError_t e = cudaSuccess;
-    std::call_once(once, []() {
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
-        cudaFuncAttributes fa{};
-        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        if (e == cudaSuccess)
-            e = cudaFuncGetAttributes(&fa, k_trsv_long);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_trsv_long, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     optin - (int)fa.sharedSizeBytes);
-    });
-    if (e != cudaSuccess)
+    static PerDevice<cudaError_t> once;
+    if (prepare_trsv(once, k_trsv_long) != cudaSuccess)
         return -1;
     const size_t smem = trsv_res_smem_bytes(a.stage_bytes, a.nstages, a.res_slots, sizeof(float));
     k_trsv_long<<<a.nblocks, kLongThreads + 32, smem, s>>>(a);

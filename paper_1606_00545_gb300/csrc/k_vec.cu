@@ -1,8 +1,7 @@
 // k_vec.cu -- vector operations (Section 2.3, Eqs. 3-6) and the fused vector
 // updates of the Krylov loops (Algorithm 4 and GMRES), each with its dot
 // products reduced in the same launch.
-#include <mutex>
-
+#include "per_device.h"
 #include "ptx.cuh"
 #include "reduce.cuh"
 
@@ -725,21 +724,23 @@ static cudaLaunchConfig_t arnoldi_config(cudaLaunchAttribute *attr, cudaStream_t
 
 template <class T> static bool arnoldi_ready()
 {
-    // a cluster of 16 is above the portable size: allowed once per process
-    static std::once_flag once;
-    static bool ok = false;
-    std::call_once(once, []() {
+    // a cluster of 16 is above the portable size: allowed once per device
+    static PerDevice<bool> once;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return once.get(dev, []() {
         cudaLaunchAttribute attr;
         const cudaLaunchConfig_t cfg = arnoldi_config(&attr, nullptr);
         int clusters = 0;
-        ok = cudaFuncSetAttribute(k_arnoldi<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                 cudaSuccess &&
-             cudaOccupancyMaxActiveClusters(&clusters, k_arnoldi<T>, &cfg) == cudaSuccess &&
-             clusters > 0;
+        const bool ok =
+            cudaFuncSetAttribute(k_arnoldi<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&clusters, k_arnoldi<T>, &cfg) == cudaSuccess &&
+            clusters > 0;
         if (!ok)
             cudaGetLastError(); // the several-launch form runs instead
+        return ok;
     });
-    return ok;
 }
 
 bool arnoldi_available(bool fp32) { return fp32 ? arnoldi_ready<float>() : arnoldi_ready<double>(); }
