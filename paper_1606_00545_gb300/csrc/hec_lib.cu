@@ -205,6 +205,7 @@ struct hec_precond_s {
     DevBuf rf_rp, rf_ci, rf_dg, rf_f, rf_src, rf_row0, rf_lev0, rf_lptr, rf_lrows, rf_plan;
     int64_t rf_nent = 0;
     int rf_longest = 0, rf_level_rows = 0; // longest factor row; mean rows of an L level (largest block)
+    int rf_largest = 0;                    // rows of the largest block
     bool rf_ready = false, factor_host_stale = false;
     int64_t device_bytes() const
     {
@@ -1306,6 +1307,7 @@ RefactorArgs refactor_args(const hec_precond_s *M)
     ra.plan = M->rf_plan.as<uint32_t>();
     ra.longest_row = M->rf_longest;
     ra.level_rows = M->rf_level_rows;
+    ra.largest_block = M->rf_largest;
     return ra;
 }
 
@@ -1322,6 +1324,7 @@ int upload_refactor_data(const hec_matrix_s *A, hec_precond_s *M, cudaStream_t s
         lev0[b + 1] = lev0[b] + (int)M->blocks[b].lptrL.size();
         nent += (int64_t)M->blocks[b].F.ci.size();
         const HostCSR &F = M->blocks[b].F;
+        M->rf_largest = std::max(M->rf_largest, F.n);
         for (int i = 0; i < F.n; ++i)
             M->rf_longest = std::max(M->rf_longest, F.rp[i + 1] - F.rp[i]);
         M->rf_level_rows = std::max(M->rf_level_rows, F.n / std::max(1, M->blocks[b].nlevL));

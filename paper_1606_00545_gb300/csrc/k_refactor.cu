@@ -459,7 +459,10 @@ static int launch_rows(const RefactorArgs &a, int nblocks, int C, cudaStream_t s
 
 int launch_refactor_plan(const RefactorArgs &a, int nblocks, cudaStream_t s)
 {
-    k_iluk_plan<kPlannedRow><<<dim3(nblocks, std::max(1, 8192 / nblocks)), kThreads, 0, s>>>(a);
+    // a thread per row, up to 8,192 CTAs
+    const int rows = (a.largest_block + kThreads - 1) / kThreads;
+    const int per = std::max(1, std::min(rows, 8192 / nblocks));
+    k_iluk_plan<kPlannedRow><<<dim3(nblocks, per), kThreads, 0, s>>>(a);
     return 0;
 }
 

@@ -274,6 +274,7 @@ struct RefactorArgs {
                              // rows of at most kPlannedRow entries)
     int longest_row;         // entries of the longest factor row
     int level_rows;          // mean rows of an L level, of the block where it is largest
+    int largest_block;       // rows of the largest block
 };
 // Per row of every chunk of a triangular-solve layout: where its values come from.
 struct FillArgs {

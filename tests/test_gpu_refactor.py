@@ -147,3 +147,29 @@ def test_refactor_zero_pivot_and_bad_handles(H):
     other = H.hec_build(A.row_ptr, A.col, A.val)
     with pytest.raises(H.HecError):
         H.hec_refactor(other, P, A.val)
+
+
+@pytest.mark.parametrize("side,k,nb", [
+    (26, 0, 1),   # planned rows (7 entries), 231 rows a level: clusters of 4
+    (36, 0, 1),   # 440 rows a level: clusters of 8
+    (20, 2, 1),   # compared columns (23 entries), 38 rows a level: one CTA
+    (48, 2, 1),   # 213 rows a level: clusters of 4
+    (60, 2, 1),   # clusters of 8
+    (24, 1, 2)])  # planned rows of 13 entries, two blocks: clusters of 2
+def test_refactor_in_clusters_bit_for_bit(H, orc, side, k, nb):
+    """Few large blocks, whose rows go to several CTAs of a cluster: the factors
+    equal those of a set-up from scratch and the oracle's, bit for bit."""
+    A0 = synth.diffusion3d_7pt_lognormal(side, 1.0, 2)
+    A1 = synth.diffusion3d_7pt_lognormal(side, 1.0, 5)
+    M = H.hec_build(A0.row_ptr, A0.col, A0.val)
+    P = H.ilu_k_setup(M, k, nb, 0)
+    H.level_schedule(P)
+    H.hec_refactor(M, P, A1.val)
+    R1 = orc.RAS(A1, k, nb, 0)
+    for b in range(nb):
+        assert np.array_equal(P.factor(b)[2], R1.block(b)[3].val), b
+    H.hec_refactor(M, P, A0.val)  # and back, by the same plan
+    M0 = H.hec_build(A0.row_ptr, A0.col, A0.val)
+    P0 = H.ilu_k_setup(M0, k, nb, 0)
+    for b in range(nb):
+        assert np.array_equal(P.factor(b)[2], P0.factor(b)[2]), b
