@@ -469,7 +469,15 @@ int launch_refactor_plan(const RefactorArgs &a, int nblocks, cudaStream_t s)
 int launch_refactor(const RefactorArgs &a, int nblocks, int sms, cudaStream_t s)
 {
     k_gather_factor<<<grid_of(a.nent), 256, 0, s>>>(a.nent, a.val, a.src, a.f);
-    if (a.longest_row > 32) { // longer rows do not fit the registers and shared memory
+    // Short rows in narrow levels have few pivots to look ahead to, and what the
+    // planned form sets up per row costs more than the merges (hec_refactor in
+    // us, merges / planned): 2D 5-point (5 entries) 200^2 in 4 blocks, 40 rows a
+    // level, 945 / 1,170; 900^2 in 4 blocks, 180 rows, 7,010 / 7,850; 500^2,
+    // 250 rows, 7,150 / 5,450; 3D 7-point (7 entries) 64^3 in 64 blocks, 95
+    // rows, 1,190 / 1,255; 40^3 in 8, 131 rows, 700 / 640; 20^3, 137 rows, 515 / 425.
+    const int narrow = a.longest_row <= 5 ? 192 : a.longest_row <= 8 ? 96 : 0;
+    // rows of more than 32 entries do not fit the registers and shared memory
+    if (a.longest_row > 32 || a.level_rows <= narrow) {
         k_iluk_numeric<<<nblocks, kThreads, 0, s>>>(a);
         return 0;
     }

@@ -173,3 +173,18 @@ def test_refactor_in_clusters_bit_for_bit(H, orc, side, k, nb):
     P0 = H.ilu_k_setup(M0, k, nb, 0)
     for b in range(nb):
         assert np.array_equal(P.factor(b)[2], P0.factor(b)[2]), b
+
+
+@pytest.mark.parametrize("side,k,nb", [(60, 0, 1), (60, 1, 3), (388, 0, 1), (380, 0, 1)])
+def test_refactor_short_rows_bit_for_bit(H, orc, side, k, nb):
+    """2D rows of 5 and 7 entries, on both sides of the level width (192 rows)
+    from which rows of 5 entries take the planned form."""
+    A0 = synth.diffusion2d_5pt_lognormal(side, 1.0, 2)
+    A1 = synth.diffusion2d_5pt_lognormal(side, 1.0, 5)
+    M = H.hec_build(A0.row_ptr, A0.col, A0.val)
+    P = H.ilu_k_setup(M, k, nb, 0)
+    H.level_schedule(P)
+    H.hec_refactor(M, P, A1.val)
+    R1 = orc.RAS(A1, k, nb, 0)
+    for b in range(nb):
+        assert np.array_equal(P.factor(b)[2], R1.block(b)[3].val), b
