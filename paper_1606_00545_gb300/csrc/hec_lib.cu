@@ -252,13 +252,15 @@ SpmvArgs spmv_args(const hec_matrix_s *A)
 // in FP32, where a thread owns four rows), at most 8 per SM.
 // With fused FP64 dots a CTA also pays a block reduction, so the CTAs take
 // equal numbers of row blocks, at most 4 CTAs per SM (75^3, two dots: 18.5 us
-// with a CTA per row block, 16.5 so; 2 per SM 19.7).
+// with a CTA per row block, 16.5 so; 2 per SM 19.7).  Not with tail rows, whose
+// sums leave row blocks of unequal times (72^3 irregular 27-point, two dots:
+// 44.9 us so, 34.7 with a CTA per row block).
 int spmv_grid(const hec_matrix_s *A, bool fp32, int ndot)
 {
     const int64_t tiles = (A->hec.n + kSpmvTile - 1) / kSpmvTile;
     const int64_t blocks = fp32 ? (tiles + 1) / 2 : tiles;
     const int grid = grid_for(blocks, 1, 8);
-    if (ndot == 0 || fp32)
+    if (ndot == 0 || fp32 || !A->hec.tail_rows.empty())
         return grid;
     const int64_t per = (blocks + 4 * device_sms() - 1) / (4 * device_sms());
     return (int)((blocks + per - 1) / per);
