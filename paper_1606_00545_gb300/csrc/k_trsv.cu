@@ -593,6 +593,7 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
         uint32_t par = 0;
         int seen0 = 0, seen1 = 0; // lane 0: the neighbours' progress seen last
         int sh = sg, pend = 0; // stage of the oldest chunk in flight; chunks in flight
+        constexpr int depth = FW > 0 ? kGatherDepth : 1; // (generic chunks: 0.5% faster so)
         // hand the oldest chunk over: its copies have landed, and lane 0 waits
         // for the neighbours' progress
         auto finish = [&]() -> bool {
@@ -629,7 +630,7 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
             const bool wait_l = g >= nL && !ldone_seen;
             // (the stage's previous chunk has been released, then its next landed)
             if (pend > 0 &&
-                (pend == kGatherDepth || wait_l ||
+                (pend == depth || wait_l ||
                  !__all_sync(0xffffffffu, (g < S || mbar_test_wait(&empty[sg], par ^ 1u)) &&
                                               mbar_test_wait(&full[sg], par)))) {
                 if (!finish()) {
@@ -1005,35 +1006,53 @@ __global__ void __launch_bounds__(kSolvers<FW> + kFeedThreads, 1) k_trsv_ras(Trs
         failed = *vfail;
 
     } else {
-        for (int c = 0; c < nch; ++c) {
-            if (!handed(s, hpar)) {
+        // The last warp, whose rows are the shortest, sees that chunk c + 1 has been
+        // handed over before chunk c's barrier (at the L pass's end after it: the
+        // U pass's right-hand sides need the whole L pass); the barrier tells the
+        // other warps.  (Every thread asking for its own chunk: 32^3 ILU(2), one
+        // block, 769 us, 753 so.)
+        const bool asks = t >= kThreads - kWarpRows;
+        auto ask = [&](int st, uint32_t par) {
+            if (asks && !handed(st, par)) {
                 err = 1;
                 *verr = 1;
             }
+        };
+        if (nch > 0)
+            ask(s, hpar);
+        if (!solvers_sync_and<NT>(!err))
+            failed = 1;
+        for (int c = 0; c < nch && !failed; ++c) {
             T out = T(0);
             T *gout = nullptr;
-            if (!err) {
-                const unsigned char *ch = stages + (size_t)s * a.stage_bytes;
-                const ChunkView<T> v = view_chunk<T>(ch);
-                if (t < v.nrows) {
-                    const bool rm = v.upass ? blk.ring_U : blk.ring_L;
-                    const T acc = solve_row_smem<T>(ch, v, t, rm, ring, v.upass ? zsc : ysc,
-                                                    rhs[(size_t)s * kThreads + t]);
-                    gout = put(v.upass, rm, v.base + t, v.upass ? v.dst[t] : -1,
-                               v.exports ? v.exp[t] : -1, acc);
-                    out = acc;
-                }
+            const unsigned char *ch = stages + (size_t)s * a.stage_bytes;
+            const ChunkView<T> v = view_chunk<T>(ch);
+            if (t < v.nrows) {
+                const bool rm = v.upass ? blk.ring_U : blk.ring_L;
+                const T acc = solve_row_smem<T>(ch, v, t, rm, ring, v.upass ? zsc : ysc,
+                                                rhs[(size_t)s * kThreads + t]);
+                gout = put(v.upass, rm, v.base + t, v.upass ? v.dst[t] : -1,
+                           v.exports ? v.exp[t] : -1, acc);
+                out = acc;
             }
+            const int s0 = s;
+            if (++s == S) {
+                s = 0;
+                hpar ^= 1u;
+            }
+            if (c + 1 < nch && c + 1 != nL)
+                ask(s, hpar);
             if (!solvers_sync_and<NT>(!err)) {
                 failed = 1; // the feeding warps' own waits run out
                 break;
             }
             if (t == kThreads - 1)
-                mbar_arrive(&empty[s]); // stage s and its right-hand-side slot are free
+                mbar_arrive(&empty[s0]); // the stage and its right-hand-side slot are free
             close(c, gout, out);
-            if (++s == S) {
-                s = 0;
-                hpar ^= 1u;
+            if (c + 1 < nch && c + 1 == nL) {
+                ask(s, hpar);
+                if (!solvers_sync_and<NT>(!err))
+                    failed = 1;
             }
         }
     }
