@@ -114,11 +114,12 @@ __global__ void __launch_bounds__(kThreads, NDOT > 0 ? 6 : TAIL ? 0 : 8) k_spmv_
     // with them in registers the kernel takes 42, 5 CTAs per SM, and the
     // gathers' latency is less well hidden.  At 40 registers, 6 CTAs per SM
     // and 4 per SM launched (see spmv_grid), the 128^3 SpMV with two dots
-    // takes 46 us (61 before, 32 without dots; the FP64 pipe alone needs 30
-    // for its 9 multiply-adds a row).  8 CTAs per SM spill: 47-51 us; the
-    // dots' partners loaded ahead of the slab: 56 us.  Without dots 32
-    // registers, 8 CTAs per SM; left to itself the compiler takes 64 for the
-    // forms with tail rows (95^3 irregular 27-point, FP32: 47 us, 41 so).
+    // takes 44 us in a row of them, 51 alone (58 and 65 before; 30 without
+    // dots; the FP64 pipe alone needs 30 for its 9 multiply-adds a row).  8
+    // CTAs per SM spill: 2 us more; the dots' partners loaded ahead of the
+    // slab: 10 more.  Without dots 32 registers, 8 CTAs per SM; left to itself
+    // the compiler takes 64 for the forms with tail rows (95^3 irregular
+    // 27-point, FP32: 47 us with 8 CTAs per SM, 41 so).
     __shared__ T s_acc[NDOT > 0 ? NDOT : 1][NDOT > 0 ? kThreads : 1];
 #pragma unroll
     for (int d = 0; d < NDOT; ++d)

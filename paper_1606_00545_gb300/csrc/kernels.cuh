@@ -221,8 +221,8 @@ struct TrsvArgs {
 // Shared memory of one CTA: stages, right-hand-side slots, own and import
 // ring, barriers and the two progress counters (vbytes: 8 for FP64, 4 for FP32).
 size_t trsv_smem_bytes(int stage_bytes, int nstages, int ring_slots, int vbytes);
-// Largest stage count (3..8) that fits the device's shared memory per CTA
-// (ring_slots: own + import slots).
+// Largest stage count (3..16) that fits the shared memory per CTA less what is
+// left free (ring_slots: own + import slots).
 int trsv_stages_for(int stage_bytes, int ring_slots, int vbytes);
 // The same for the resident-vector kernel: stages and a vector of res_slots values.
 size_t trsv_res_smem_bytes(int stage_bytes, int nstages, int res_slots, int vbytes);

@@ -433,10 +433,10 @@ bool set_thresholds(const BlockFactor &B, BlockPlan &bp, int RI)
             }
         }
     }
-    // The kernel completes chunk k only after chunks k + 1 and k + 2 of the
-    // same pass have been handed over too (the first is loaded, the second
-    // confirmed, before chunk k's barrier), so completing k needs all three
-    // chunks' thresholds met.
+    // The kernel completes chunk k only after chunk k + 1 of the same pass has
+    // been handed over too (it is loaded before chunk k's barrier).  Here chunk
+    // k + 2's thresholds are asked for as well: more than a split needs, so that
+    // a split that is planned runs with a chunk to spare.
     std::vector<int> done(P, 0);
     auto met = [&](int p, const ChunkPlan &ch) {
         return ch.need_prev <= (p > 0 ? done[p - 1] : 0) &&
@@ -1199,8 +1199,10 @@ int pack_trsv(const std::vector<BlockFactor> &Bs, int n, int stage_bytes, int ma
         return HEC_ERR_INVALID;
     }
     const int nb = (int)Bs.size();
-    // fixed-slot chunks carry export slots whenever blocks may be split, and
-    // a stage holds the largest one (the kernel reads every warp's slots)
+    // fixed-slot chunks carry export slots whenever blocks may be split; they
+    // are planned against a stage that holds a full one (the stage launched is
+    // the largest chunk emitted: the kernel reads no slot past a chunk's last
+    // warp)
     const bool exps = parts > 1;
     if (uniform_width > 0) {
         if (uniform_width > kNarrowRow) {
